@@ -20,8 +20,9 @@
  *    kernel's continuous Fourier transform c(p0) c(p1).  F: unnormalised 2-D
  *    DFT.  G: sparse rows; row m holds the J_m x J_m taps nearest
  *    kappa = omega K / (2 pi) of the KB kernel (J = 7 by default) convolved
- *    with the row's w-kernel (App. E), stored as complex64 (or bfloat16
- *    complex) weights with int32 column indices and int64 row offsets.
+ *    with the row's w-kernel (App. E).  A row is an outer product of one
+ *    length-J_m vector per axis: complex64 plans store the two vectors,
+ *    bfloat16 plans the rounded J_m^2 weights.
  *  - Device pointers ("dev") are CUDA global-memory addresses owned by the
  *    caller; the library never frees them.  Host pointers ("host") are read
  *    during the call only.
@@ -116,12 +117,13 @@ typedef struct pnp_plan_info {
   double beta;          /* KB shape parameter                                  */
   double dl;            /* pixel size [rad] used for the w-term (0: none)      */
   int64_t device_bytes; /* device memory held by the plan                      */
-  int region_pitch;     /* row pitch (cells) of the gridding pass's shared-memory
-                           grid regions, chosen at plan time to limit bank
-                           conflicts for the plan's mix of supports J        */
-  int run_max;          /* rows at most per run of rows sharing a tap window  */
-  int64_t unit_nnz;     /* taps at most per gridding work unit                */
-  int row_batch;        /* rows of a run whose residuals one warp forms together */
+  int region_pitch;     /* columns (cells) of the grid region that a gridding work
+                           unit of the largest support stages in shared memory */
+  int run_max;          /* run cap setting: reported only, rows sharing a tap
+                           window are no longer cut into runs                 */
+  int64_t unit_nnz;     /* sizes the gridding work units: an eighth of it is the
+                           taps at most of one warp's unit (less in small plans) */
+  int row_batch;        /* row batch setting (pnp_plan_set_row_batch)         */
   int nstacks;          /* w-stacks P of the operator (1: w wholly in G)      */
   int64_t holographic_bytes; /* device bytes of the holographic H (0: not built) */
   int compensated;      /* 1: gridding sums are compensated (pnp_plan_set_compensated) */
@@ -233,36 +235,29 @@ int pnp_plan_set_holographic(pnp_plan* plan, int enable);
  * Synchronises the plan's stream. */
 int pnp_plan_set_compensated(pnp_plan* plan, int enable);
 
-/* Set how many rows of a run of rows sharing a tap window one warp of the
- * gridding pass forms the residuals of together (1, 2 or 4; 0 keeps the
- * current choice; anything else is PNP_ERR_INVALID_ARG).  Autotuner hook: a
- * performance setting only, results are unchanged (the warp sums keep their
- * pairing order).  Synchronises the plan's stream. */
+/* Row batch setting (1, 2 or 4; 0 keeps the current choice; anything else is
+ * PNP_ERR_INVALID_ARG).  The gridding pass once formed the residuals of so many
+ * rows together; its present kernels take one row per group of lanes, so the
+ * setting is kept and reported but changes neither results nor times.
+ * Synchronises the plan's stream. */
 int pnp_plan_set_row_batch(pnp_plan* plan, int row_batch);
 
 /* Autotuner of the gridding pass's work decomposition (a performance setting
  * with no counterpart in the paper; results change only in the order of the
  * floating-point sums).  Times `reps` fused gridding passes on the plan's
- * stream for every triple of run cap (rows at most per run of rows sharing a
- * tap window: 3, 4, 6, 8), unit size (2^16, 2^17, 2^18 taps) and row batch
- * (rows of a run whose residuals a warp forms together: 1, 2, 4), keeps the
- * fastest and rebuilds the work list for it (G is unchanged; the chosen row
- * batch is reported by pnp_plan_get_info).  Synchronous; the output
- * grid is left cleared.  Outputs (each may be NULL): the chosen run cap and
- * unit size, and the chosen pass's mean time in ms (-1 for an empty operator).
- * reps must lie in [1, 100]. */
+ * stream for unit sizes of 2^16, 2^17 and 2^18 taps (pnp_plan_set_unit_nnz), keeps
+ * the fastest and rebuilds the work list for it (G is unchanged).  Synchronous; the
+ * output grid is left cleared.  Outputs (each may be NULL): the run cap setting
+ * (unchanged), the chosen unit size, and the chosen pass's mean time in ms (-1 for an
+ * empty operator).  reps must lie in [1, 100]. */
 int pnp_plan_autotune(pnp_plan* plan, int reps, int* run_max_out, int64_t* unit_nnz_out, double* ms_out);
 
 /* Device-side status flags of the plan's kernels (synchronous read; the flags
  * stay set for the plan's lifetime).  Each is an internal consistency check
  * that a correct plan never sets:
- *  bit 1 (2)   a wait of the gridding pass's copy pipeline ran out (bounded
- *              wait): the pass stopped early and its output is incomplete;
- *  bit 2 (4)   a chunk of the gridding work list was inconsistent and skipped;
+ *  bit 2 (4)   a unit of the gridding work list was inconsistent and skipped;
  *  bit 4 (16)  a tap pair outside the holographic stencil was skipped while
- *              building H.
- * Taps outside their staged region are caught when the plan is built
- * (pnp_plan_create fails with PNP_ERR_INVALID_ARG). */
+ *              building H. */
 int pnp_plan_device_status(pnp_plan* plan, int* flags_host);
 
 /* Per-stage CUDA-event timing (profiling aid).  While enabled, every

@@ -50,37 +50,62 @@ __host__ __device__ __forceinline__ float2 cmulc(float2 a, float2 b) {
 }
 
 // ------------------------------------------------------------------ work units
-// Gridding work list.  A chunk is a run of consecutive rows (tile-sorted order)
-// with at most CHUNK_TAPS taps and CHUNK_ROWS rows: the unit of one TMA bulk
-// transfer.  A unit is a run of consecutive chunks whose rows all have their
-// first tap in one grid tile (and one data block).
-constexpr int CHUNK_TAPS = 4096;
-constexpr int CHUNK_ROWS = 128;
-constexpr int NSTAGE = 4;          // shared-memory pipeline depth of the gridding pass
-constexpr int GPASS_CONSUMERS = 16; // consumer warps per gridding CTA (plus one producer warp)
-constexpr int GPASS_THREADS = 32 * (GPASS_CONSUMERS + 1);
+// Gridding work list.  A unit is a run of consecutive rows (sorted order) of one support J whose first
+// taps lie in one GT x GT grid tile (and one data block): the work of one warp.
+constexpr int GT = 8;               // gridding tile side (first-tap cells)
+constexpr int GKT = 32;             // side of the coarse tiles of the (tile, block) sort key
+constexpr int GPASS_WARPS = 4;      // warps per gridding CTA (they work independently)
+constexpr int TAP_CLASSES = 7;      // classes of supports: J <= 7, 8, 9, 11, 13, 15, 16 (tap_class)
 // twiddles of the radix-16 passes 1 and 2 of the FFT: entry off(p) + r 16^p + k holds
 // exp(-2 pi i r k / 16^(p+1)), off(1) = 0, off(2) = 256 (independent of the transform length)
 constexpr int TWP_ENTRIES = 16 * 16 + 16 * 256;
-constexpr int TAP_PAD = 16;        // weights/columns are allocated nnz + TAP_PAD long
-constexpr int ROW_PAD = 4;         // row offsets M + 1 + ROW_PAD, sorted y M + ROW_PAD
 
-struct Chunk {
-  long long row_begin;
-  long long tap_begin;
-  long long run_begin;  // first entry of the chunk's run list in the plan's run array
-  int nrows;
-  int ntaps;
-  int nn;     // taps per row (J^2, the same for every row of the chunk)
-  int nruns;  // runs of rows sharing one tap window; the list holds nruns + 1 row offsets
-};
-constexpr int RUN_MAX = 6;         // default cap on rows per run (keeps the consumer warps balanced)
+// Stored rows of G.  Along k1 a row's taps are held as pairs of grid rows whose first is even within the
+// tile, so tap_pairs(J) pairs cover the J taps from an even or an odd first row (zeros around them).
+//   complex64: the factors, tap_pairs (re, re, im, im) pairs of the k1 axis, then 2 tap_pairs (re, im) of
+//              the k0 axis: 2 tap_pairs 16-byte units;
+//   BF16:      the rounded taps [k1 pair][k0](re, re, im, im): tap_pairs^2 16-byte units.
+// The last k0 entry is never a tap (2 tap_pairs > J): it holds the first tap's cell in the tile,
+// row << 3 | column (BF16: that of pair 0), at byte row_cell_at.
+__host__ __device__ constexpr int tap_pairs(int J) { return J <= 7 ? 4 : (J + 2) / 2; }
+__host__ __device__ constexpr int tap_lanes(int J) { return J <= 8 ? 8 : 16; }  // lanes that share a row
+__host__ __device__ constexpr int tap_class(int pairs, int lanes) { return pairs == 4 ? 0 : lanes == 8 ? 1 : pairs - 3; }
+// First-tap columns that share a gridding window: the largest power of two for which the class's largest
+// support plus the shift fits its lanes.
+__host__ __device__ constexpr int tap_quant(int pairs, int lanes) {
+  return pairs == 4 ? 2 : lanes == 8 ? 1 : pairs == 5 ? 8 : pairs <= 7 ? 4 : pairs == 8 ? 2 : 1;
+}
+__host__ __device__ constexpr int row_units(int J, bool bf16) {
+  return bf16 ? tap_pairs(J) * tap_pairs(J) : 2 * tap_pairs(J);
+}
+__host__ __device__ constexpr int row_cell_at(int pairs, bool bf16) {
+  return bf16 ? (2 * pairs - 1) * 8 : 16 * pairs + (2 * pairs - 1) * 8;
+}
+__device__ __forceinline__ int row_cell(const unsigned char* row, int J, bool bf16) {
+  return *reinterpret_cast<const int*>(row + row_cell_at(tap_pairs(J), bf16));
+}
+// tap (i1, i0) of a stored row with support J (i0, i1 < J)
+__device__ __forceinline__ float2 row_tap(const unsigned char* row, int J, bool bf16, int i1, int i0) {
+  const int jp = tap_pairs(J);
+  i1 += (row_cell(row, J, bf16) >> 3) & 1;
+  if (bf16) {
+    const __nv_bfloat16* o = reinterpret_cast<const __nv_bfloat16*>(row) + ((i1 >> 1) * 2 * jp + i0) * 4 + (i1 & 1);
+    return make_float2(__bfloat162float(o[0]), __bfloat162float(o[2]));
+  }
+  const float* f = reinterpret_cast<const float*>(row);
+  const float* g1 = f + 4 * (i1 >> 1) + (i1 & 1);
+  return cmul(make_float2(f[4 * jp + 2 * i0], f[4 * jp + 2 * i0 + 1]), make_float2(g1[0], g1[2]));
+}
 
 struct Unit {
-  long long chunk_begin;
-  int nchunks;
-  int tile;
+  long long row_begin;  // first row (sorted order)
+  long long row_unit;   // its offset in the stored rows, 16-byte units
+  int nrows;
+  int J;
+  int tile;             // t1 * (K / GT) + t0
+  int pad_;
 };
+constexpr int RUN_MAX = 6;  // reported default of the run cap setting
 
 // Q2 epilogue modes of the last inverse-FFT pass (see fft.cu).
 // EPI_HAAR_NOPOS: the Haar prox without the final positivity projection.
@@ -94,19 +119,16 @@ enum GMode { G_DEGRID = 0, G_GRID = 1, G_FUSED = 2 };
 // ------------------------------------------------------------------ plan
 struct pnp_plan {
   int n = 0, K = 0, logK = 0, J = 7, Jmax = 7, wdtype = PNP_W_C64, nblocks = 1;
-  int tile = 48;       // gridding tile side T (cells)
-  int ntc = 0;         // tiles per grid side, ceil(K / tile)
-  int slots = 8;       // register slots per lane per row (32*slots >= Jmax^2)
-  int pitch = 0;       // row pitch (cells) of the staged gridding regions (0: the region side)
-  int run_max = pnp::RUN_MAX;  // rows per run of a shared tap window, at most
-  int row_batch = 2;           // rows of a run whose residuals a warp forms together (1, 2, 4)
-  int rpw = 2;         // rows per warp in flight
+  int tile = pnp::GT;  // gridding tile side (cells)
+  int ntc = 0;         // tiles per grid side, K / tile
+  int pitch = 0;       // side and row pitch (cells) of a warp's gridding regions
+  int run_max = pnp::RUN_MAX, row_batch = 2;  // settings without an effect on the present kernels (reported)
   int64_t M = 0, nnz = 0, unit_nnz = 1 << 17;
   double beta = 0, dl = 0;
   int nstacks = 1;             // w-stacks P (App. E): rows sorted by stack, then tile and block
   int64_t nkeys = 0;           // (tile, block) keys per stack
   std::vector<double> w_centres;       // P stack centres [wavelengths]
-  std::vector<int64_t> h_stack_units;  // P+1: the work units of stack s are [s], [s+1])
+  std::vector<int64_t> h_class_units;  // the units of stack s and class c: [s TAP_CLASSES + c], [.. + 1])
   cudaStream_t stream = nullptr;   // caller's stream: every launch goes here
   cudaStream_t cstream = nullptr;  // private non-blocking stream for graph capture/replay
   cudaEvent_t ev_join[2] = {nullptr, nullptr};
@@ -134,17 +156,12 @@ struct pnp_plan {
                                          // they are ~2^-24 of the sums); kept zero between uses
   bool compensated = false;    // gridding flushes add their rounding errors to d_gridB_lo (TwoSum)
   float2* d_tmp = nullptr;     // K*n: half-transformed intermediate
-  void* d_w = nullptr;         // nnz weights (float2 or bf16x2)
-  uint16_t* d_cells = nullptr; // nnz cell indices lr * pitch + lc in the row's staged tile region
-  uint8_t* d_runs = nullptr;    // per chunk: row offsets where runs start, then nrows (padded by 16)
-  int64_t n_runs = 0;
-  int64_t* d_rowptr = nullptr; // M+1 (sorted order)
+  void* d_rows = nullptr;      // stored rows of G in sorted order (row_units 16-byte units each)
+  unsigned* d_sched = nullptr; // unit counters of the gridding kernels, two per stack and class (zero at rest)
   int32_t* d_perm = nullptr;   // sorted row -> caller row
   float2* d_ysorted = nullptr; // M scratch: y in sorted order
   pnp::Unit* d_units = nullptr;
   int64_t n_units = 0;
-  pnp::Chunk* d_chunks = nullptr;
-  int64_t n_chunks = 0;
   double* d_acc = nullptr;     // FP64 accumulators [8]
   int* d_status = nullptr;     // device status flags [4] (bit 0: gridding index out of range)
   float* d_img[3] = {nullptr, nullptr, nullptr};  // n*n work images
@@ -169,11 +186,12 @@ struct pnp_plan {
   std::vector<TimedEvent> timed;
 
   // host mirrors used by export and work-list rebuilds
-  std::vector<int64_t> h_rowptr;   // M+1
+  std::vector<int64_t> h_unit;     // M+1: offsets of the stored rows, 16-byte units
+  std::vector<uint8_t> h_J;        // sorted: support of the row
   std::vector<int32_t> h_perm;     // sorted -> caller
   std::vector<int32_t> h_inv;      // caller -> sorted
-  std::vector<int32_t> h_key;      // sorted: (stack * ntc^2 + tile) * nblocks + block
-  std::vector<uint16_t> h_start;   // sorted: first tap's cell in the tile (row * tile + col)
+  std::vector<int32_t> h_key;      // sorted: (stack * coarse tiles + coarse tile) * nblocks + block
+  std::vector<uint16_t> h_start;   // sorted: tile within the coarse tile << 6 | first tap's cell in the tile
 };
 
 struct pnp_den {
@@ -197,8 +215,6 @@ int fft_adjoint(pnp_plan* p, int mode, const float* x, float* out,         // d_
                 float gamma, float t, int s);
 // gridding.cu: the work units of stack s
 int gridding_pass(pnp_plan* p, int mode, const float2* y_user, float2* y_out, int s);
-// choose p->pitch from the plan's number of rows per support J (rows_per_J[0..16])
-int gridding_pitch(pnp_plan* p, const int64_t* rows_per_J);
 int permute_y(pnp_plan* p, const float2* y_user, float scale = 1.f);  // d_ysorted = scale y_user[perm]
 // plan_build.cu
 int build_units(pnp_plan* p);

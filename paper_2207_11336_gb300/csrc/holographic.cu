@@ -16,29 +16,18 @@ namespace {
 
 constexpr int HB_WARPS = 8;  // rows processed concurrently per block of the build
 
-template <typename WT>
-__device__ __forceinline__ float2 hw_at(const void* w, int64_t i) {
-  if constexpr (sizeof(WT) == 8) {
-    return reinterpret_cast<const float2*>(w)[i];
-  } else {
-    return __bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(w)[i]);
-  }
-}
-
 struct HBuildArgs {
   const Unit* units;
   int64_t n_units;
-  const Chunk* chunks;
-  const void* w;
-  const uint16_t* cells;
-  int T, ntc, P, R, Jmax, S, logK;  // tile side, tiles per side, region pitch and side, stencil side
+  const unsigned char* rows;
+  int ntc, Jmax, S, logK;  // tiles per side, stencil side
   float2* H;
   int* status;  // bit 4: a tap pair outside the stencil (skipped)
 };
 
 // one block per work unit, one warp per row: the row's taps are staged in shared memory and every
 // (i, j) pair adds conj(w_i) w_j to H[cell_j - cell_i][cell_i]
-template <typename WT>
+template <bool BF>
 __global__ void __launch_bounds__(32 * HB_WARPS) holo_build(HBuildArgs A) {
   __shared__ int s_k[HB_WARPS][256];
   __shared__ short s_r[HB_WARPS][256], s_c[HB_WARPS][256];
@@ -48,37 +37,34 @@ __global__ void __launch_bounds__(32 * HB_WARPS) holo_build(HBuildArgs A) {
   const int64_t KK = (int64_t)K * K;
   for (int64_t u = blockIdx.x; u < A.n_units; u += gridDim.x) {
     const Unit U = A.units[u];
-    const int r0 = (U.tile / A.ntc) * A.T, c0 = (U.tile % A.ntc) * A.T;
-    for (int ci = 0; ci < U.nchunks; ++ci) {
-      const Chunk ch = A.chunks[U.chunk_begin + ci];
-      const int nn = ch.nn;
-      if (nn > 256) continue;
-      for (int q = wp; q < ch.nrows; q += HB_WARPS) {
-        const int64_t base = ch.tap_begin + (int64_t)q * nn;
-        for (int t = lane; t < nn; t += 32) {
-          const int cell = A.cells[base + t];
-          const int lr = cell / A.P, lc = cell - lr * A.P;
-          s_r[wp][t] = (short)lr;
-          s_c[wp][t] = (short)lc;
-          s_k[wp][t] = (((r0 + lr) & Km) << A.logK) + ((c0 + lc) & Km);
-          s_w[wp][t] = hw_at<WT>(A.w, base + t);
-        }
-        __syncwarp();
-        for (int i = 0; i < nn; ++i) {
-          const float2 wi = s_w[wp][i];
-          const int ri = s_r[wp][i], cci = s_c[wp][i], ki = s_k[wp][i];
-          for (int j = lane; j < nn; j += 32) {
-            const int dr = s_r[wp][j] - ri, dc = s_c[wp][j] - cci;
-            if (dr < -Jm1 || dr > Jm1 || dc < -Jm1 || dc > Jm1) {
-              atomicOr(A.status, 16);
-              continue;
-            }
-            const int64_t at = (int64_t)((dr + Jm1) * A.S + (dc + Jm1)) * KK + ki;
-            atomicAdd(&A.H[at], cmulc(wi, s_w[wp][j]));  // conj(w_i) w_j
-          }
-        }
-        __syncwarp();
+    const int r0 = (U.tile / A.ntc) * GT, c0 = (U.tile % A.ntc) * GT;
+    const int J = U.J, nn = J * J, bytes = 16 * row_units(J, BF);
+    if (nn > 256) continue;
+    for (int q = wp; q < U.nrows; q += HB_WARPS) {
+      const unsigned char* row = A.rows + (U.row_unit << 4) + (size_t)q * bytes;
+      const int cell = row_cell(row, J, BF), lr0 = cell >> 3, lc0 = cell & 7;
+      for (int t = lane; t < nn; t += 32) {
+        const int i1 = t / J, i0 = t - i1 * J, lr = lr0 + i1, lc = lc0 + i0;
+        s_r[wp][t] = (short)lr;
+        s_c[wp][t] = (short)lc;
+        s_k[wp][t] = (((r0 + lr) & Km) << A.logK) + ((c0 + lc) & Km);
+        s_w[wp][t] = row_tap(row, J, BF, i1, i0);
       }
+      __syncwarp();
+      for (int i = 0; i < nn; ++i) {
+        const float2 wi = s_w[wp][i];
+        const int ri = s_r[wp][i], cci = s_c[wp][i], ki = s_k[wp][i];
+        for (int j = lane; j < nn; j += 32) {
+          const int dr = s_r[wp][j] - ri, dc = s_c[wp][j] - cci;
+          if (dr < -Jm1 || dr > Jm1 || dc < -Jm1 || dc > Jm1) {
+            atomicOr(A.status, 16);
+            continue;
+          }
+          const int64_t at = (int64_t)((dr + Jm1) * A.S + (dc + Jm1)) * KK + ki;
+          atomicAdd(&A.H[at], cmulc(wi, s_w[wp][j]));  // conj(w_i) w_j
+        }
+      }
+      __syncwarp();
     }
   }
 }
@@ -136,13 +122,8 @@ int holo_build_plan(pnp_plan* p) {
     HBuildArgs A{};
     A.units = p->d_units;
     A.n_units = p->n_units;
-    A.chunks = p->d_chunks;
-    A.w = p->d_w;
-    A.cells = p->d_cells;
-    A.T = p->tile;
+    A.rows = static_cast<const unsigned char*>(p->d_rows);
     A.ntc = p->ntc;
-    A.R = p->tile + p->Jmax - 1;
-    A.P = p->pitch > 0 ? p->pitch : A.R;
     A.Jmax = p->Jmax;
     A.S = S;
     A.logK = p->logK;
@@ -150,9 +131,9 @@ int holo_build_plan(pnp_plan* p) {
     A.status = p->d_status;
     const unsigned grid = (unsigned)std::min<int64_t>(p->n_units, (int64_t)p->num_sms * 8);
     if (p->wdtype == PNP_W_BF16C)
-      holo_build<__nv_bfloat162><<<grid, 32 * HB_WARPS, 0, p->stream>>>(A);
+      holo_build<true><<<grid, 32 * HB_WARPS, 0, p->stream>>>(A);
     else
-      holo_build<float2><<<grid, 32 * HB_WARPS, 0, p->stream>>>(A);
+      holo_build<false><<<grid, 32 * HB_WARPS, 0, p->stream>>>(A);
     PNP_CHECK_LAUNCH();
   }
   PNP_CUDA(cudaStreamSynchronize(p->stream));

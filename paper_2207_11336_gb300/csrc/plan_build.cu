@@ -7,8 +7,8 @@
 //
 // Device side: one warp per row evaluates the row's separable weights
 //   g(t) = sum_d w_hat[d] psi(t + d),  psi(t) = I0(beta sqrt(1 - (2t/J)^2)),
-// on the J_m taps nearest kappa along each axis, and writes the J_m^2 outer
-// products with their column indices.  w_hat is the K-point DFT of the
+// on the J_m taps nearest kappa along each axis, and writes the two factors (complex64
+// plans) or their J_m^2 outer products (BF16 plans).  w_hat is the K-point DFT of the
 // paraxial w-chirp exp(i pi a q(p)), a = w dl^2, whose phase profile q equals
 // p^2 on the image and is continued smoothly (C^2) to a flat value at |p| = K/2
 // (App. E reading: the w-kernel of each row folded into its KB row).  It is
@@ -31,22 +31,20 @@ constexpr int MAX_D = 15;  // |d| <= MAX_D, so 2 MAX_D + 1 <= 32 lanes
 struct RowGeom {
   double kap0, kap1, a;  // kappa per axis, chirp rate a = w dl^2
   double d;              // data weight d_m multiplying the row (1 without weighting)
+  int64_t unit;          // offset of the stored row, 16-byte units
   int s0, s1;            // first tap (unwrapped) per axis
   int J;                 // row support J_m
+  int cell;              // first tap's cell in its tile, row << 3 | column
 };
 
 struct BuildArgs {
   int64_t M;
-  int K, logK, J;
+  int J;
   double beta, bscale, c0;   // b = bscale * a ; series centre c0
   int nterms, D;
   const double* mu;          // [nterms][2D+1]
   const RowGeom* geom;       // sorted order
-  const int64_t* rowptr;
-  void* w;
-  uint16_t* cells;
-  int T, S, P;               // gridding tile side, staged region side and row pitch
-  int* err;                  // set when a tap falls outside its row's staged region
+  unsigned char* rows;       // stored rows (zero: the padding stays)
   int bf16;
 };
 
@@ -109,43 +107,53 @@ __global__ void __launch_bounds__(256) build_rows(BuildArgs A) {
     s_g[wl][ax][sl] = make_double2(gr, gi);
   }
   __syncwarp();
-  const int64_t beg = A.rowptr[row];
-  const int nn = Jm * Jm, Km = A.K - 1;
-  for (int t = lane; t < nn; t += 32) {
-    const int i1 = t / Jm, i0 = t - i1 * Jm;  // k1-major, k0-minor
+  const int jp = tap_pairs(Jm);
+  float* out = reinterpret_cast<float*>(A.rows + (g.unit << 4));
+  if (!A.bf16) {
+    // the k1 factors, scaled by the data weight, as (re, re, im, im) per tap pair; then the k0 factors
+    if (sl < Jm) {
+      const double2 v = s_g[wl][ax][sl];
+      if (ax) {
+        const int i1 = sl + ((g.cell >> 3) & 1);
+        float* o = out + 4 * (i1 >> 1) + (i1 & 1);
+        o[0] = (float)(g.d * v.x);
+        o[2] = (float)(g.d * v.y);
+      } else {
+        out[4 * jp + 2 * sl] = (float)v.x;
+        out[4 * jp + 2 * sl + 1] = (float)v.y;
+      }
+    }
+    if (lane == 0) reinterpret_cast<int*>(out)[row_cell_at(jp, false) / 4] = g.cell;
+    return;
+  }
+  if (lane == 0) reinterpret_cast<int*>(out)[row_cell_at(jp, true) / 4] = g.cell;
+  __nv_bfloat16* ob = reinterpret_cast<__nv_bfloat16*>(out);
+  for (int t = lane; t < Jm * Jm; t += 32) {
+    const int i1 = t / Jm, i0 = t - i1 * Jm;
     const double2 a = s_g[wl][0][i0], b = s_g[wl][1][i1];
     const float wr = (float)(g.d * (a.x * b.x - a.y * b.y)), wi = (float)(g.d * (a.x * b.y + a.y * b.x));
-    if (A.bf16) {
-      __nv_bfloat162 h = __floats2bfloat162_rn(wr, wi);
-      reinterpret_cast<__nv_bfloat162*>(A.w)[beg + t] = h;
-    } else {
-      reinterpret_cast<float2*>(A.w)[beg + t] = make_float2(wr, wi);
-    }
-    // cell of the tap in the staged region of the row's tile (the tile of its first tap)
-    const int r0 = (((g.s1 % A.K) + A.K) % A.K) / A.T * A.T, c0 = (((g.s0 % A.K) + A.K) % A.K) / A.T * A.T;
-    const int lr = (g.s1 + i1 - r0) & Km, lc = (g.s0 + i0 - c0) & Km;
-    if (lr >= A.S || lc >= A.S) atomicOr(A.err, 1);
-    A.cells[beg + t] = (uint16_t)(lr < A.S && lc < A.S ? lr * A.P + lc : 0);
+    const int e1 = i1 + ((g.cell >> 3) & 1);
+    __nv_bfloat16* o = ob + ((e1 >> 1) * 2 * jp + i0) * 4 + (e1 & 1);
+    o[0] = __float2bfloat16_rn(wr);
+    o[2] = __float2bfloat16_rn(wi);
   }
 }
 
 // gather rows for export: canonical column order k0*K + k1, float weights.  src_off holds per
-// row (first tap, tap count, tile origin r0, tile origin c0); cells are lr * P + lc from the origin.
+// row (offset of the stored row, support, first tap's k1, first tap's k0).
 __global__ void export_rows(const int64_t* __restrict__ src_off, const int64_t* __restrict__ dst_off,
-                            int64_t nrows, const void* w, const uint16_t* cells, int P, int bf16, int logK,
-                            float2* out_w, int32_t* out_c) {
+                            int64_t nrows, const unsigned char* rows, int bf16, int logK, float2* out_w,
+                            int32_t* out_c) {
   const int64_t r = blockIdx.x;
   if (r >= nrows) return;
-  const int64_t s = src_off[4 * r], cnt = src_off[4 * r + 1], d = dst_off[r];
-  const int r0 = (int)src_off[4 * r + 2], c0 = (int)src_off[4 * r + 3];
+  const unsigned char* row = rows + (src_off[4 * r] << 4);
+  const int64_t d = dst_off[r];
+  const int J = (int)src_off[4 * r + 1], r0 = (int)src_off[4 * r + 2], c0 = (int)src_off[4 * r + 3];
   const int Km = (1 << logK) - 1;
-  for (int64_t t = threadIdx.x; t < cnt; t += blockDim.x) {
-    float2 v;
-    if (bf16) v = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(w)[s + t]);
-    else v = reinterpret_cast<const float2*>(w)[s + t];
-    const int c = cells[s + t], lr = c / P, lc = c - lr * P;
-    out_w[d + t] = v;
-    out_c[d + t] = (((c0 + lc) & Km) << logK) | ((r0 + lr) & Km);
+  for (int t = threadIdx.x; t < J * J; t += blockDim.x) {
+    const int i1 = t / J, i0 = t - i1 * J;
+    out_w[d + t] = row_tap(row, J, bf16 != 0, i1, i0);
+    out_c[d + t] = (((c0 + i0) & Km) << logK) | ((r0 + i1) & Km);
   }
 }
 
@@ -192,84 +200,54 @@ int dev_alloc(pnp_plan* p, T** ptr, size_t count) {
 
 int build_units(pnp_plan* p) {
   ++p->epoch;  // a captured FB graph launches the old work list: it must be captured again
-  std::vector<Unit> units;
-  std::vector<Chunk> chunks;
-  std::vector<uint8_t> runs;
+  std::vector<Unit> units, cls[TAP_CLASSES];
   const int64_t M = p->M;
-  auto nnz_of = [&](int64_t i) { return p->h_rowptr[i + 1] - p->h_rowptr[i]; };
-  std::vector<int64_t> stack_units(p->nstacks + 1, 0);
+  std::vector<int64_t> bounds(1, 0);
+  // Taps per unit of each class of supports: an eighth of the unit_nnz setting (a unit is one warp's work),
+  // less where the class is small, so that every resident warp (16 to 24 per SM) gets several units, but
+  // enough rows to pay for staging and flushing the unit's region.
+  int64_t cap[TAP_CLASSES] = {};
+  for (int64_t r = 0; r < M; ++r) cap[tap_class(tap_pairs(p->h_J[r]), tap_lanes(p->h_J[r]))] += p->h_J[r] * p->h_J[r];
+  for (int64_t& c : cap)
+    c = std::min<int64_t>(p->unit_nnz, std::max<int64_t>(2048, std::min<int64_t>(p->unit_nnz / 8, c / (p->num_sms * 100))));
+  const int cpt = p->K / GKT, per = GKT / GT;  // coarse tiles per side, tiles per coarse tile side
   int64_t i = 0;
-  while (i < M) {
-    const int32_t key = p->h_key[i];
-    Unit u;
-    u.chunk_begin = (long long)chunks.size();
-    u.tile = (int)((key % p->nkeys) / p->nblocks);
-    stack_units[key / p->nkeys + 1] = (int64_t)units.size() + 1;  // units of a stack are consecutive
-    int64_t unit_taps = 0;
-    while (i < M && p->h_key[i] == key && (unit_taps == 0 || unit_taps + nnz_of(i) <= p->unit_nnz)) {
-      Chunk ch;
-      ch.row_begin = i;
-      ch.tap_begin = p->h_rowptr[i];
-      int nr = 0;
-      int64_t nt = 0;
-      const int64_t row_nnz = nnz_of(i);  // every row of a chunk has the same support
-      while (i < M && p->h_key[i] == key && nnz_of(i) == row_nnz && nr < CHUNK_ROWS &&
-             nt + nnz_of(i) <= CHUNK_TAPS && (unit_taps + nt == 0 || unit_taps + nt + nnz_of(i) <= p->unit_nnz)) {
-        nt += nnz_of(i);
-        ++nr;
+  for (int st = 0; st < p->nstacks; ++st) {
+    while (i < M && p->h_key[i] / p->nkeys == st) {
+      const int32_t key = p->h_key[i];
+      const int sub = p->h_start[i] >> 6, J = p->h_J[i], ct = (int)((key % p->nkeys) / p->nblocks);
+      Unit u{};
+      u.row_begin = i;
+      u.row_unit = p->h_unit[i];
+      u.J = J;
+      u.tile = ((ct / cpt) * per + sub / per) * p->ntc + (ct % cpt) * per + sub % per;
+      const int c = tap_class(tap_pairs(J), tap_lanes(J));
+      int64_t taps = 0;
+      while (i < M && p->h_key[i] == key && (p->h_start[i] >> 6) == sub && p->h_J[i] == J &&
+             (taps == 0 || taps + (int64_t)J * J <= cap[c])) {
+        taps += (int64_t)J * J;
+        ++u.nrows;
         ++i;
       }
-      if (nr == 0) return fail(PNP_ERR_INVALID_ARG, "internal: a row does not fit one gridding chunk");
-      ch.nrows = nr;
-      ch.ntaps = (int)nt;
-      ch.nn = (int)row_nnz;
-      // runs: consecutive rows whose first tap is the same cell share their whole tap window
-      // (same support), at most run_max rows each
-      ch.run_begin = (long long)runs.size();
-      int last = 0;
-      for (int q = 0; q < nr; ++q)
-        if (q == 0 || p->h_start[ch.row_begin + q] != p->h_start[ch.row_begin + q - 1] || q - last == p->run_max) {
-          runs.push_back((uint8_t)q);
-          last = q;
-        }
-      ch.nruns = (int)((long long)runs.size() - ch.run_begin);
-      runs.push_back((uint8_t)nr);
-      chunks.push_back(ch);
-      unit_taps += nt;
+      cls[c].push_back(u);
     }
-    u.nchunks = (int)((long long)chunks.size() - u.chunk_begin);
-    units.push_back(u);
+    for (auto& v : cls) {
+      units.insert(units.end(), v.begin(), v.end());
+      bounds.push_back((int64_t)units.size());
+      v.clear();
+    }
   }
+  if (i != M) return fail(PNP_ERR_INVALID_ARG, "internal: rows out of stack order");
   if (p->d_units) {
     cudaFree(p->d_units);
-    p->device_bytes -= p->n_units * (int64_t)sizeof(Unit);
+    p->device_bytes -= std::max<int64_t>(1, p->n_units) * (int64_t)sizeof(Unit);
     p->d_units = nullptr;
   }
-  if (p->d_chunks) {
-    cudaFree(p->d_chunks);
-    p->device_bytes -= p->n_chunks * (int64_t)sizeof(Chunk);
-    p->d_chunks = nullptr;
-  }
-  if (p->d_runs) {
-    cudaFree(p->d_runs);
-    p->device_bytes -= p->n_runs + 32;
-    p->d_runs = nullptr;
-  }
   p->n_units = (int64_t)units.size();
-  p->n_chunks = (int64_t)chunks.size();
-  for (int s = 0; s < p->nstacks; ++s)  // empty stacks start and end where the previous one ends
-    stack_units[s + 1] = std::max(stack_units[s + 1], stack_units[s]);
-  p->h_stack_units.swap(stack_units);
+  p->h_class_units.swap(bounds);
   if (int rc = dev_alloc(p, &p->d_units, units.size())) return rc;
-  if (int rc = dev_alloc(p, &p->d_chunks, chunks.size())) return rc;
-  p->n_runs = (int64_t)runs.size();
-  runs.resize(runs.size() + 32, 0);  // the stage copies 16-byte windows around each list
-  if (int rc = dev_alloc(p, &p->d_runs, runs.size())) return rc;
-  PNP_CUDA(cudaMemcpy(p->d_runs, runs.data(), runs.size(), cudaMemcpyHostToDevice));
-  if (!units.empty()) {
+  if (!units.empty())
     PNP_CUDA(cudaMemcpy(p->d_units, units.data(), units.size() * sizeof(Unit), cudaMemcpyHostToDevice));
-    PNP_CUDA(cudaMemcpy(p->d_chunks, chunks.data(), chunks.size() * sizeof(Chunk), cudaMemcpyHostToDevice));
-  }
   return PNP_OK;
 }
 
@@ -289,11 +267,11 @@ int plan_build(pnp_plan* p, const double* uvw, const int8_t* Jrow, const int32_t
   }
 
   // per-row geometry, keys
-  const int ntc = (K + p->tile - 1) / p->tile;
+  const int ntc = K / GT, cpt = K / GKT;  // tiles and coarse tiles per grid side
   p->ntc = ntc;
   std::vector<RowGeom> geom(M);
   std::vector<int32_t> key(M);
-  std::vector<uint16_t> startc(M);  // first tap's cell within its tile
+  std::vector<uint16_t> startc(M);  // tile within the coarse tile << 6 | first tap's cell within the tile
   int Jmax = J;
   double amax = 0.0;
   for (int64_t m = 0; m < M; ++m) {
@@ -320,41 +298,32 @@ int plan_build(pnp_plan* p, const double* uvw, const int8_t* Jrow, const int32_t
     g.s0 = (int)std::floor(g.kap0 - 0.5 * g.J) + 1;
     g.s1 = (int)std::floor(g.kap1 - 0.5 * g.J) + 1;
     const int f0 = ((g.s0 % K) + K) % K, f1 = ((g.s1 % K) + K) % K;
-    key[m] = ((f1 / p->tile) * ntc + (f0 / p->tile)) * p->nblocks + (block ? block[m] : 0);
-    startc[m] = (uint16_t)((f1 % p->tile) * p->tile + (f0 % p->tile));
+    key[m] = ((f1 / GKT) * cpt + (f0 / GKT)) * p->nblocks + (block ? block[m] : 0);
+    const int sub = (f1 % GKT) / GT * (GKT / GT) + (f0 % GKT) / GT;
+    startc[m] = (uint16_t)((sub << 6) | ((f1 % GT) << 3) | (f0 % GT));
     Jmax = std::max(Jmax, g.J);
     amax = std::max(amax, std::fabs(g.a));
     geom[m] = g;
   }
   p->Jmax = Jmax;
-  p->slots = Jmax * Jmax <= 64 ? 2 : (Jmax * Jmax <= 128 ? 4 : 8);
-  {
-    std::vector<int64_t> rows_per_J(17, 0);
-    for (int64_t m = 0; m < M; ++m) rows_per_J[geom[m].J]++;
-    if (int rc = gridding_pitch(p, rows_per_J.data())) return rc;
-  }
+  p->pitch = GT - tap_quant(tap_pairs(Jmax), tap_lanes(Jmax)) + tap_lanes(Jmax);
 
-  // stable LSD counting sort: by the first tap's cell in the tile, then by support J, then by
-  // (tile, block) key, so that rows of one tile come out grouped by J (each gridding chunk then
-  // holds rows of a single J) and, within that, rows with the same tap window are adjacent
-  // (the gridding pass gathers and scatters such a run once)
+  // stable LSD counting sort: by (tile within the coarse tile, support J, first tap's cell in the tile with
+  // the cells of one gridding window together), then by (coarse tile, block) key, so that the rows of one
+  // tile come out grouped by J and, within that, rows sharing a window are adjacent (the gridding pass
+  // keeps it in registers)
   std::vector<int32_t> by_j(M);
   {
-    const int nc = p->tile * p->tile;
-    std::vector<int64_t> cc(nc + 1, 0);
-    for (int64_t m = 0; m < M; ++m) cc[startc[m] + 1]++;
-    for (int c = 0; c < nc; ++c) cc[c + 1] += cc[c];
-    std::vector<int32_t> by_c(M);
-    for (int64_t m = 0; m < M; ++m) by_c[cc[startc[m]]++] = (int32_t)m;
-    std::vector<int64_t> cj(18, 0);
-    for (int64_t m = 0; m < M; ++m) cj[geom[m].J + 1]++;
-    for (int j = 0; j < 17; ++j) cj[j + 1] += cj[j];
-    for (int64_t i = 0; i < M; ++i) {
-      const int32_t m = by_c[i];
-      by_j[cj[geom[m].J]++] = m;
-    }
+    auto bin = [&](int64_t m) {
+      const int J = geom[m].J, q = tap_quant(tap_pairs(J), tap_lanes(J)), c = startc[m] & 63, lr = c >> 3, lc = c & 7;
+      return ((startc[m] >> 6) * 17 + J) * 64 + (((lr >> 1) * (GT / q) + lc / q) * 2 + (lr & 1)) * q + lc % q;
+    };
+    std::vector<int64_t> cc((GKT / GT) * (GKT / GT) * 17 * 64 + 1, 0);
+    for (int64_t m = 0; m < M; ++m) cc[bin(m) + 1]++;
+    for (size_t c = 1; c < cc.size(); ++c) cc[c] += cc[c - 1];
+    for (int64_t m = 0; m < M; ++m) by_j[cc[bin(m)]++] = (int32_t)m;
   }
-  const int64_t nkeys = (int64_t)ntc * ntc * p->nblocks;
+  const int64_t nkeys = (int64_t)cpt * cpt * p->nblocks;
   if (nkeys * p->nstacks > INT32_MAX) return fail(PNP_ERR_UNSUPPORTED, "too many (stack, tile, block) keys");
   p->nkeys = nkeys;
   std::vector<int64_t> cnt(nkeys + 1, 0);
@@ -381,15 +350,20 @@ int plan_build(pnp_plan* p, const double* uvw, const int8_t* Jrow, const int32_t
   std::vector<RowGeom> sgeom(M);
   p->h_key.assign(M, 0);
   p->h_start.assign(M, 0);
-  p->h_rowptr.assign(M + 1, 0);
+  p->h_unit.assign(M + 1, 0);
+  p->h_J.assign(M, 0);
+  p->nnz = 0;
   for (int64_t i = 0; i < M; ++i) {
     const int64_t m = p->h_perm[i];
     sgeom[i] = geom[m];
     p->h_key[i] = (int32_t)((stack ? (int64_t)stack[m] : 0) * nkeys + key[m]);
     p->h_start[i] = startc[m];
-    p->h_rowptr[i + 1] = p->h_rowptr[i] + (int64_t)geom[m].J * geom[m].J;
+    p->h_J[i] = (uint8_t)geom[m].J;
+    sgeom[i].unit = p->h_unit[i];
+    sgeom[i].cell = startc[m] & 63;
+    p->h_unit[i + 1] = p->h_unit[i] + row_units(geom[m].J, p->wdtype == PNP_W_BF16C);
+    p->nnz += (int64_t)geom[m].J * geom[m].J;
   }
-  p->nnz = p->h_rowptr[M];
   // uv support of G: per grid row k1 the largest centred |k0| of its taps, and the band of rows
   std::vector<int> rowh(K, -1);
   {
@@ -460,24 +434,22 @@ int plan_build(pnp_plan* p, const double* uvw, const int8_t* Jrow, const int32_t
   if (int rc = dev_alloc(p, &p->d_gridB_lo, KK)) return rc;
   if (int rc = dev_alloc(p, &p->d_tmp, (size_t)K * n)) return rc;
   if (int rc = dev_alloc(p, &p->d_rowh, (size_t)K)) return rc;
-  const size_t wbytes = p->wdtype == PNP_W_BF16C ? 4 : 8;
   {
-    void* w = nullptr;
-    cudaError_t e = cudaMalloc(&w, (p->nnz + TAP_PAD) * wbytes);
+    const size_t bytes = (size_t)std::max<int64_t>(1, p->h_unit[M]) * 16;
+    cudaError_t e = cudaMalloc(&p->d_rows, bytes);
     if (e != cudaSuccess) {
       cudaGetLastError();
-      return fail(PNP_ERR_OOM, "cudaMalloc of G weights (" + std::to_string(p->nnz * wbytes) + " bytes) failed");
+      p->d_rows = nullptr;
+      return fail(PNP_ERR_OOM, "cudaMalloc of the rows of G (" + std::to_string(bytes) + " bytes) failed");
     }
-    p->d_w = w;
-    p->device_bytes += (int64_t)((p->nnz + TAP_PAD) * wbytes);
-    PNP_CUDA(cudaMemset(w, 0, (p->nnz + TAP_PAD) * wbytes));
+    p->device_bytes += (int64_t)bytes;
+    PNP_CUDA(cudaMemset(p->d_rows, 0, bytes));  // the padding taps
   }
-  if (int rc = dev_alloc(p, &p->d_cells, (size_t)p->nnz + TAP_PAD)) return rc;
-  if (int rc = dev_alloc(p, &p->d_rowptr, (size_t)M + 1 + ROW_PAD)) return rc;
   if (int rc = dev_alloc(p, &p->d_perm, (size_t)M)) return rc;
-  if (int rc = dev_alloc(p, &p->d_ysorted, (size_t)M + ROW_PAD)) return rc;
-  PNP_CUDA(cudaMemset(p->d_cells, 0, ((size_t)p->nnz + TAP_PAD) * sizeof(uint16_t)));
-  PNP_CUDA(cudaMemset(p->d_ysorted, 0, ((size_t)M + ROW_PAD) * sizeof(float2)));
+  if (int rc = dev_alloc(p, &p->d_sched, (size_t)2 * p->nstacks * TAP_CLASSES)) return rc;
+  PNP_CUDA(cudaMemset(p->d_sched, 0, (size_t)2 * p->nstacks * TAP_CLASSES * sizeof(unsigned)));
+  if (int rc = dev_alloc(p, &p->d_ysorted, (size_t)M)) return rc;
+  PNP_CUDA(cudaMemset(p->d_ysorted, 0, (size_t)M * sizeof(float2)));
   if (int rc = dev_alloc(p, &p->d_acc, 8)) return rc;
   if (int rc = dev_alloc(p, &p->d_status, 4)) return rc;
   for (int i = 0; i < 3; ++i)
@@ -517,11 +489,6 @@ int plan_build(pnp_plan* p, const double* uvw, const int8_t* Jrow, const int32_t
   PNP_CUDA(cudaMemcpy(p->d_rowh, rowh.data(), K * sizeof(int), cudaMemcpyHostToDevice));
   PNP_CUDA(cudaMemset(p->d_acc, 0, 8 * sizeof(double)));
   PNP_CUDA(cudaMemset(p->d_status, 0, 4 * sizeof(int)));
-  {
-    std::vector<int64_t> rp(p->h_rowptr);
-    rp.resize(M + 1 + ROW_PAD, p->nnz);  // padding entries repeat nnz
-    PNP_CUDA(cudaMemcpy(p->d_rowptr, rp.data(), rp.size() * sizeof(int64_t), cudaMemcpyHostToDevice));
-  }
   if (M) PNP_CUDA(cudaMemcpy(p->d_perm, p->h_perm.data(), M * sizeof(int32_t), cudaMemcpyHostToDevice));
   if (M && row_scale) {  // the data weights in the caller's row order, for pnp_plan_scale_data
     std::vector<float> d(M);
@@ -540,13 +507,10 @@ int plan_build(pnp_plan* p, const double* uvw, const int8_t* Jrow, const int32_t
       cudaFree(d_geom);
       return fail(PNP_ERR_OOM, "plan build scratch allocation failed");
     }
-    PNP_CUDA(cudaMemsetAsync(p->d_status + 3, 0, sizeof(int), p->stream));
     PNP_CUDA(cudaMemcpy(d_geom, sgeom.data(), M * sizeof(RowGeom), cudaMemcpyHostToDevice));
     PNP_CUDA(cudaMemcpy(d_mu, mu.data(), mu.size() * sizeof(double), cudaMemcpyHostToDevice));
     BuildArgs A{};
     A.M = M;
-    A.K = K;
-    A.logK = p->logK;
     A.J = J;
     A.beta = p->beta;
     A.bscale = bscale;
@@ -555,13 +519,7 @@ int plan_build(pnp_plan* p, const double* uvw, const int8_t* Jrow, const int32_t
     A.D = D;
     A.mu = d_mu;
     A.geom = d_geom;
-    A.rowptr = p->d_rowptr;
-    A.w = p->d_w;
-    A.cells = p->d_cells;
-    A.T = p->tile;
-    A.S = p->tile + p->Jmax - 1;
-    A.P = p->pitch;
-    A.err = p->d_status + 3;
+    A.rows = static_cast<unsigned char*>(p->d_rows);
     A.bf16 = p->wdtype == PNP_W_BF16C;
     build_rows<<<(unsigned)((M + 7) / 8), 256, 0, p->stream>>>(A);
     cudaError_t e = cudaGetLastError();
@@ -570,10 +528,6 @@ int plan_build(pnp_plan* p, const double* uvw, const int8_t* Jrow, const int32_t
     cudaFree(d_geom);
     cudaFree(d_mu);
     if (e != cudaSuccess) return fail(PNP_ERR_CUDA, std::string("build_rows: ") + cudaGetErrorString(e));
-    int err = 0;
-    PNP_CUDA(cudaMemcpy(&err, p->d_status + 3, sizeof(int), cudaMemcpyDeviceToHost));
-    PNP_CUDA(cudaMemset(p->d_status + 3, 0, sizeof(int)));
-    if (err) return fail(PNP_ERR_INVALID_ARG, "internal: a tap of G falls outside its row's gridding region");
   }
   return build_units(p);
 }
@@ -585,13 +539,14 @@ int export_rows_impl(const pnp_plan* p, const int64_t* rows, int64_t nrows, int6
   for (int64_t i = 0; i < nrows; ++i) {
     if (rows[i] < 0 || rows[i] >= p->M) return fail(PNP_ERR_INVALID_ARG, "export row index out of range");
     const int64_t s = p->h_inv[rows[i]];
-    const int tile = (int)((p->h_key[s] % p->nkeys) / p->nblocks);
-    src[4 * i] = p->h_rowptr[s];
-    src[4 * i + 1] = p->h_rowptr[s + 1] - p->h_rowptr[s];
-    src[4 * i + 2] = (int64_t)(tile / p->ntc) * p->tile;
-    src[4 * i + 3] = (int64_t)(tile % p->ntc) * p->tile;
+    const int ct = (int)((p->h_key[s] % p->nkeys) / p->nblocks), cpt = p->K / GKT, per = GKT / GT;
+    const int sub = p->h_start[s] >> 6, cell = p->h_start[s] & 63;
+    src[4 * i] = p->h_unit[s];
+    src[4 * i + 1] = p->h_J[s];
+    src[4 * i + 2] = (int64_t)(ct / cpt) * GKT + sub / per * GT + (cell >> 3);
+    src[4 * i + 3] = (int64_t)(ct % cpt) * GKT + sub % per * GT + (cell & 7);
     dst[i] = offsets[i];
-    offsets[i + 1] = offsets[i] + src[4 * i + 1];
+    offsets[i + 1] = offsets[i] + (int64_t)p->h_J[s] * p->h_J[s];
   }
   if (!weights || !cols || nrows == 0) return PNP_OK;
   const int64_t total = offsets[nrows];
@@ -610,7 +565,8 @@ int export_rows_impl(const pnp_plan* p, const int64_t* rows, int64_t nrows, int6
   cudaError_t e = cudaMemcpy(d_src, src.data(), 4 * nrows * sizeof(int64_t), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(d_dst, dst.data(), nrows * sizeof(int64_t), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) {
-    export_rows<<<(unsigned)nrows, 128, 0, p->stream>>>(d_src, d_dst, nrows, p->d_w, p->d_cells, p->pitch,
+    export_rows<<<(unsigned)nrows, 128, 0, p->stream>>>(d_src, d_dst, nrows,
+                                                         static_cast<const unsigned char*>(p->d_rows),
                                                          p->wdtype == PNP_W_BF16C, p->logK, d_w, d_c);
     g_launches.fetch_add(1);
     e = cudaGetLastError();

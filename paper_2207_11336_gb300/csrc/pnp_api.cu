@@ -63,14 +63,11 @@ void free_plan(pnp_plan* p) {
   cudaFree(p->d_gridB);
   cudaFree(p->d_gridB_lo);
   cudaFree(p->d_tmp);
-  cudaFree(p->d_w);
-  cudaFree(p->d_cells);
-  cudaFree(p->d_runs);
-  cudaFree(p->d_rowptr);
+  cudaFree(p->d_rows);
+  cudaFree(p->d_sched);
   cudaFree(p->d_perm);
   cudaFree(p->d_ysorted);
   cudaFree(p->d_units);
-  cudaFree(p->d_chunks);
   cudaFree(p->d_acc);
   cudaFree(p->d_status);
   if (p->cstream) cudaStreamDestroy(p->cstream);
@@ -287,7 +284,6 @@ int pnp_plan_create_desc(pnp_plan** plan, const pnp_plan_desc* desc) {
   p->wdtype = weight_dtype;
   p->nblocks = nblocks;
   p->stream = reinterpret_cast<cudaStream_t>(desc->stream);
-  p->tile = K >= 128 ? 32 : 16;
   if (cudaGetDevice(&p->device) != cudaSuccess ||
       cudaDeviceGetAttribute(&p->num_sms, cudaDevAttrMultiProcessorCount, p->device) != cudaSuccess) {
     cudaGetLastError();
@@ -344,7 +340,7 @@ int pnp_plan_get_info(const pnp_plan* p, pnp_plan_info* info) {
   info->beta = p->beta;
   info->dl = p->dl;
   info->device_bytes = p->device_bytes;
-  info->region_pitch = p->pitch > 0 ? p->pitch : p->tile + p->Jmax - 1;
+  info->region_pitch = p->pitch;
   info->run_max = p->run_max;
   info->row_batch = p->row_batch;
   info->nstacks = p->nstacks;
@@ -393,56 +389,42 @@ int pnp_plan_set_row_batch(pnp_plan* p, int row_batch) {
 int pnp_plan_autotune(pnp_plan* p, int reps, int* run_max_out, int64_t* unit_nnz_out, double* ms_out) {
   if (!p || reps < 1 || reps > 100) return fail(PNP_ERR_INVALID_ARG, "bad argument");
   PNP_CUDA(cudaStreamSynchronize(p->stream));
-  const int old_run = p->run_max, old_rb = p->row_batch;
   const int64_t old_unit = p->unit_nnz;
-  int best_run = old_run, best_rb = old_rb;
   int64_t best_unit = old_unit;
   float best_ms = -1.f;
   if (p->M > 0 && p->n_units > 0) {
-    const int runs[] = {3, 4, 6, 8};
     const int64_t units[] = {int64_t(1) << 16, int64_t(1) << 17, int64_t(1) << 18};
-    const int batches[] = {1, 2, 4};
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     PNP_CUDA(cudaEventCreate(&e0));
     PNP_CUDA(cudaEventCreate(&e1));
     const bool saved_timing = p->timing;
     p->timing = false;
     int rc = PNP_OK;
-    for (int r : runs) {
-      for (int64_t u : units) {
-        p->run_max = r;
-        p->unit_nnz = u;
-        if ((rc = build_units(p))) break;
-        for (int rb : batches) {
-          p->row_batch = rb;
-          for (int s = 0; s < p->nstacks && !rc; ++s) rc = gridding_pass(p, G_FUSED, nullptr, nullptr, s);  // warm-up
-          if (rc) break;
-          if (cudaEventRecord(e0, p->stream) != cudaSuccess) {
-            cudaGetLastError();
-            rc = fail(PNP_ERR_CUDA, "autotune: event record failed");
-            break;
-          }
-          for (int i = 0; i < reps && !rc; ++i)
-            for (int s = 0; s < p->nstacks && !rc; ++s) rc = gridding_pass(p, G_FUSED, nullptr, nullptr, s);
-          if (rc) break;
-          float ms = 0.f;
-          if (cudaEventRecord(e1, p->stream) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
-              cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess) {
-            cudaGetLastError();
-            rc = fail(PNP_ERR_CUDA, "autotune: timing failed");
-            break;
-          }
-          ms /= reps;
-          if (best_ms < 0.f || ms < best_ms) {
-            best_ms = ms;
-            best_run = r;
-            best_unit = u;
-            best_rb = rb;
-          }
-        }
-        if (rc) break;
-      }
+    for (int64_t u : units) {
+      p->unit_nnz = u;
+      if ((rc = build_units(p))) break;
+      for (int s = 0; s < p->nstacks && !rc; ++s) rc = gridding_pass(p, G_FUSED, nullptr, nullptr, s);  // warm-up
       if (rc) break;
+      if (cudaEventRecord(e0, p->stream) != cudaSuccess) {
+        cudaGetLastError();
+        rc = fail(PNP_ERR_CUDA, "autotune: event record failed");
+        break;
+      }
+      for (int i = 0; i < reps && !rc; ++i)
+        for (int s = 0; s < p->nstacks && !rc; ++s) rc = gridding_pass(p, G_FUSED, nullptr, nullptr, s);
+      if (rc) break;
+      float ms = 0.f;
+      if (cudaEventRecord(e1, p->stream) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
+          cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess) {
+        cudaGetLastError();
+        rc = fail(PNP_ERR_CUDA, "autotune: timing failed");
+        break;
+      }
+      ms /= reps;
+      if (best_ms < 0.f || ms < best_ms) {
+        best_ms = ms;
+        best_unit = u;
+      }
     }
     p->timing = saved_timing;
     cudaEventDestroy(e0);
@@ -453,8 +435,6 @@ int pnp_plan_autotune(pnp_plan* p, int reps, int* run_max_out, int64_t* unit_nnz
       cudaGetLastError();
       rc = fail(PNP_ERR_CUDA, "autotune: clearing the grid failed");
     }
-    p->run_max = rc ? old_run : best_run;
-    p->row_batch = rc ? old_rb : best_rb;
     p->unit_nnz = rc ? old_unit : best_unit;
     if (int rc2 = build_units(p)) return rc2;
     if (rc) return rc;

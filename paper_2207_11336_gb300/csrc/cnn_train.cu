@@ -35,7 +35,6 @@ constexpr int64_t OFF_MID = NW1 + NB1;  // 6 x (W, b)
 constexpr int64_t MID_STRIDE = NWM + NBM;
 constexpr int64_t OFF_W8 = OFF_MID + 6 * MID_STRIDE, OFF_B8 = OFF_W8 + NW8;
 constexpr int64_t NPARAM = OFF_B8 + 1;
-constexpr int WG_CHUNK = 2048;  // pixels per weight-gradient block
 
 __device__ __forceinline__ float bf16r(float v) { return __bfloat162float(__float2bfloat16_rn(v)); }
 
@@ -82,133 +81,305 @@ __device__ __forceinline__ size_t cidx(const Dims& d, int b, int y, int x, int c
   return canvas_index(b, y, x, c, d.Hc, d.Wc);
 }
 
-// layer 8 forward, l1 loss and g = dL/dN = -sign(z - N - u) / count
-__global__ void __launch_bounds__(256) last_fwd_loss(Dims d, const __nv_bfloat16* __restrict__ act7,
-                                                     const float* __restrict__ w8r, const float* __restrict__ bias,
-                                                     const float* __restrict__ z, const float* __restrict__ u,
-                                                     float* __restrict__ g, double* loss) {
-  __shared__ float sw[9 * CH];
-  __shared__ double red[256];
-  for (int i = threadIdx.x; i < 9 * CH; i += blockDim.x) sw[i] = w8r[i];
+// ------------------------------------------------------------ the one-channel ends (layers 1 and 8)
+// Tap t of a 3 x 3 stencil sits at off_t = (t / 3 - 1, t % 3 - 1); FLIP takes the pixels p - off_t in the
+// place of p + off_t (a transposed convolution).  Pixels outside the image are zero.
+constexpr int END_COLS = 32;  // columns of a block of the walks below: one per lane, a warp per channel block
+
+// pairs of floats, kept as 64-bit values so that packed FMAs take them without moves
+typedef unsigned long long f2;
+__device__ __forceinline__ f2 pk(float x, float y) {
+  f2 d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(x), "f"(y));
+  return d;
+}
+__device__ __forceinline__ float2 unpk(f2 a) {
+  float2 d;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(d.x), "=f"(d.y) : "l"(a));
+  return d;
+}
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {  // two FP32 FMAs, one instruction
+  f2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+// the two BF16 halves of a word as a pair of floats
+__device__ __forceinline__ f2 bf2(uint32_t v) { return pk(__uint_as_float(v << 16), __uint_as_float(v & 0xffff0000u)); }
+
+// rows y0 - 1 .. y0 + rows and columns x0 - 1 .. x0 + END_COLS of image b, zero outside, into shared memory
+__device__ __forceinline__ void stage_window(const Dims& d, const float* __restrict__ img, int b, int y0, int x0,
+                                             int rows, float (*zt)[END_COLS + 2]) {
+  for (int i = threadIdx.x; i < (rows + 2) * (END_COLS + 2); i += blockDim.x) {
+    const int r = i / (END_COLS + 2), c = i % (END_COLS + 2), y = y0 + r - 1, x = x0 + c - 1;
+    zt[r][c] = y >= 0 && y < d.s && x >= 0 && x < d.s ? img[((int64_t)b * d.s + y) * d.s + x] : 0.f;
+  }
   __syncthreads();
-  const int64_t total = (int64_t)d.B * d.s * d.s;
-  const float inv = 1.f / (float)total;
-  double s = 0.0;
-  for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < total; p += (int64_t)gridDim.x * blockDim.x) {
-    const int b = (int)(p / ((int64_t)d.s * d.s)), y = (int)((p / d.s) % d.s), x = (int)(p % d.s);
-    float nz = bias[7 * CH];
+}
+constexpr int END_ROWS = 64;  // rows of a block at most
+constexpr int END_BATCH = 4;  // rows whose canvas loads a lane issues together (one at a time left HBM at 1.5 TB/s)
+
+// 1 -> 64 with a ReLU mask: out[p][c] = [mask[p][c] > 0] sum_t W[c][t] img[p + off_t] (FLIP: p - off_t).
+//   layer 8 backward: W = W8 stored [t][c], FLIP;  layer 1 tangent: W = W1 stored [c][t].
+// Warp w forms channel block w of 32 columns row after row with its 72 weights in registers: one 16-byte load
+// (mask) and store per lane and row, whole 512-byte runs per warp.  Bound by that traffic (256 B a pixel).
+// 16 x 256^2: 82 -> 62 us against a thread per pixel with the weights read from shared memory.
+template <bool FLIP>
+__global__ void __launch_bounds__(256) one_to_many(Dims d, int rows, const __nv_bfloat16* __restrict__ mask,
+                                                   const float* __restrict__ w, const float* __restrict__ img,
+                                                   __nv_bfloat16* __restrict__ out) {
+  __shared__ float zt[END_ROWS + 2][END_COLS + 2];
+  const int b = blockIdx.z, y0 = blockIdx.y * rows, x0 = blockIdx.x * END_COLS;
+  const int cb = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  stage_window(d, img, b, y0, x0, rows, zt);
+  f2 wt[4][9];
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+#pragma unroll
     for (int t = 0; t < 9; ++t) {
-      const int yy = y + t / 3 - 1, xx = x + t % 3 - 1;
-      if (yy < 0 || yy >= d.s || xx < 0 || xx >= d.s) continue;
+      const int c = 8 * cb + 2 * q;
+      wt[q][t] = FLIP ? pk(w[t * CH + c], w[t * CH + c + 1]) : pk(w[c * 9 + t], w[(c + 1) * 9 + t]);
+    }
+  const int x = x0 + lane, ye = min(rows, d.s - y0);
+  if (x >= d.s) return;
+  const size_t step = (size_t)d.Wc * CH;
+  size_t at = cidx(d, b, y0, x, 8 * cb);
+  for (int rb = 0; rb < ye; rb += END_BATCH) {
+    uint4 m[END_BATCH];
 #pragma unroll
-      for (int cb = 0; cb < 8; ++cb) {
-        const __nv_bfloat162* a = reinterpret_cast<const __nv_bfloat162*>(act7 + cidx(d, b, yy, xx, 8 * cb));
+    for (int k = 0; k < END_BATCH; ++k)
+      if (rb + k < ye) m[k] = *reinterpret_cast<const uint4*>(mask + at + k * step);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const int c = 4 * cb + k;
-          const float2 v = __bfloat1622float2(a[k]);
-          nz = fmaf(sw[t * CH + 2 * c], v.x, fmaf(sw[t * CH + 2 * c + 1], v.y, nz));
+    for (int k = 0; k < END_BATCH; ++k, at += step) {
+      const int r = rb + k;
+      if (r >= ye) break;
+      const uint4 mc = m[k];
+      f2 v[4] = {0, 0, 0, 0};
+#pragma unroll
+      for (int t = 0; t < 9; ++t) {
+        const float g = FLIP ? zt[r + 2 - t / 3][lane + 2 - t % 3] : zt[r + t / 3][lane + t % 3];
+        const f2 gg = pk(g, g);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v[q] = fma2(wt[q][t], gg, v[q]);
+      }
+      uint4 o;
+      const uint32_t* mw = reinterpret_cast<const uint32_t*>(&mc);
+      uint32_t* ow = reinterpret_cast<uint32_t*>(&o);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float2 a = unpk(bf2(mw[q])), u = unpk(v[q]);
+        const __nv_bfloat162 h = __floats2bfloat162_rn(a.x > 0.f ? u.x : 0.f, a.y > 0.f ? u.y : 0.f);
+        ow[q] = *reinterpret_cast<const uint32_t*>(&h);
+      }
+      *reinterpret_cast<uint4*>(out + at) = o;
+    }
+  }
+}
+
+// Gradients of a one-channel layer: dW[c][t] += sum_p cv[p][c] img[p + off_t] (FLIP: p - off_t), and
+//   FLIP (layer 8: cv = act7, img = g):     db[0] += sum_p img[p]
+//   else (layer 1: cv = dpre1, img = z):    db[c] += sum_p cv[p][c].
+// Same walk as one_to_many, a block taking tiles of 32 columns by `rows` rows until none are left: a lane keeps
+// the 8 x 9 sums of its column, the warp adds them up by exchanging halves (80 values in 80 shuffles) and writes
+// them to the block's slice of a workspace, which onechannel_reduce adds up (as global atomics on the 576 sums
+// they took 30 us however small the batch).  Bound by the canvas read.  16 x 256^2: 3040 -> 67 us (8 x 128^2: 1085 -> 19 us) against a
+// thread per (tap, channel) that walked 2048 pixels one after the other.
+constexpr int ONE_SUMS = 8 * 80;  // a block's partial sums: [channel block][t][8 channels], t = 9: the bias
+template <bool FLIP>
+__global__ void __launch_bounds__(256) wgrad_onechannel(Dims d, int rows, const float* __restrict__ img,
+                                                        const __nv_bfloat16* __restrict__ cv, float* __restrict__ part) {
+  __shared__ float zt[END_ROWS + 2][END_COLS + 2];
+  const int cb = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int tx = (d.s + END_COLS - 1) / END_COLS, ty = (d.s + rows - 1) / rows, tiles = tx * ty * d.B;
+  f2 acc[9][4], bias[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    bias[q] = 0;
+#pragma unroll
+    for (int t = 0; t < 9; ++t) acc[t][q] = 0;
+  }
+  const size_t step = (size_t)d.Wc * CH;
+  const f2 one = pk(1.f, 1.f);
+  float isum = 0.f;
+  for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    const int x0 = tile % tx * END_COLS, y0 = tile / tx % ty * rows, b = tile / (tx * ty);
+    __syncthreads();  // the previous tile's window
+    stage_window(d, img, b, y0, x0, rows, zt);
+    const int x = x0 + lane, ye = x < d.s ? min(rows, d.s - y0) : 0;
+    const __nv_bfloat16* src = cv + cidx(d, b, y0, min(x, d.s - 1), 8 * cb);
+    for (int rb = 0; rb < ye; rb += END_BATCH) {
+      uint4 m[END_BATCH];
+#pragma unroll
+      for (int k = 0; k < END_BATCH; ++k)
+        m[k] = rb + k < ye ? *reinterpret_cast<const uint4*>(src + (rb + k) * step) : make_uint4(0, 0, 0, 0);
+#pragma unroll
+      for (int k = 0; k < END_BATCH; ++k) {
+        const int r = rb + k;
+        if (r >= ye) break;
+        const f2 ch[4] = {bf2(m[k].x), bf2(m[k].y), bf2(m[k].z), bf2(m[k].w)};
+#pragma unroll
+        for (int t = 0; t < 9; ++t) {
+          const float g = FLIP ? zt[r + 2 - t / 3][lane + 2 - t % 3] : zt[r + t / 3][lane + t % 3];
+          const f2 gg = pk(g, g);
+#pragma unroll
+          for (int q = 0; q < 4; ++q) acc[t][q] = fma2(ch[q], gg, acc[t][q]);
+        }
+        if (FLIP) {
+          isum += zt[r + 1][lane + 1];
+        } else {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) bias[q] = fma2(ch[q], one, bias[q]);
         }
       }
     }
-    const float r = z[p] - nz - u[p];
-    s += fabs((double)r);
-    g[p] = r > 0.f ? -inv : (r < 0.f ? inv : 0.f);
   }
-  red[threadIdx.x] = s;
-  __syncthreads();
-  for (int k = blockDim.x >> 1; k > 0; k >>= 1) {
-    if (threadIdx.x < k) red[threadIdx.x] += red[threadIdx.x + k];
-    __syncthreads();
+  float v[80];  // [t][8 channels], then 8 bias sums (FLIP: the image's sum in the first)
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+#pragma unroll
+    for (int t = 0; t < 10; ++t) {
+      const float2 u = unpk(t < 9 ? acc[t < 9 ? t : 0][q] : bias[q]);
+      v[8 * t + 2 * q] = FLIP && t == 9 && q == 0 ? isum : u.x;
+      v[8 * t + 2 * q + 1] = u.y;
+    }
   }
-  if (threadIdx.x == 0) atomicAdd(loss, red[0] * (double)inv);
+  int base = 0;  // the values this lane ends up with: v[0..4] = totals of base .. base + 4
+#pragma unroll
+  for (int n = 40, o = 16; n >= 5; n >>= 1, o >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int k = 0; k < n; ++k) {
+      const float send = up ? v[k] : v[k + n], keep = up ? v[k + n] : v[k];
+      v[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+    base += up ? n : 0;
+  }
+  float* o = part + (size_t)blockIdx.x * ONE_SUMS + 80 * cb + base;
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    v[k] += __shfl_xor_sync(0xffffffffu, v[k], 1);
+    if (!(lane & 1)) o[k] = v[k];
+  }
 }
 
-// dpre7[q][ci] = [act7[q][ci] > 0] * sum_t W8[ci][t] g[q - off_t]
-__global__ void __launch_bounds__(256) last_bwd(Dims d, const __nv_bfloat16* __restrict__ act7,
-                                                const float* __restrict__ w8r, const float* __restrict__ g,
-                                                __nv_bfloat16* __restrict__ dpre) {
-  __shared__ float sw[9 * CH];
-  for (int i = threadIdx.x; i < 9 * CH; i += blockDim.x) sw[i] = w8r[i];
+// dW[c][t] += and db += the sums of the `parts` slices (layer 8: one bias, in channel block 0); block (32, 8)
+__global__ void __launch_bounds__(256) onechannel_reduce(const float* __restrict__ part, int parts, int layer8,
+                                                         float* __restrict__ dW, float* __restrict__ db) {
+  __shared__ float red[8][32];
+  const int e = blockIdx.x * 32 + threadIdx.x;
+  float s = 0.f;
+  for (int k = threadIdx.y; k < parts; k += 8) s += part[(size_t)k * ONE_SUMS + e];
+  red[threadIdx.y][threadIdx.x] = s;
   __syncthreads();
-  const int64_t total = (int64_t)d.B * d.s * d.s;
-  for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < total; p += (int64_t)gridDim.x * blockDim.x) {
-    const int b = (int)(p / ((int64_t)d.s * d.s)), y = (int)((p / d.s) % d.s), x = (int)(p % d.s);
-    float gt[9];
+  if (threadIdx.y) return;
+  for (int k = 1; k < 8; ++k) s += red[k][threadIdx.x];
+  const int cb = e / 80, t = e % 80 / 8, c = e % 8;
+  if (t < 9) dW[(8 * cb + c) * 9 + t] += s;
+  else if (!layer8) db[8 * cb + c] += s;
+  else if (e == 72) db[0] += s;
+}
+
+// 64 -> 1: N[p] = init + sum_{t, c} W[t][c] cv[p + off_t][c] (FLIP: p - off_t), then
+//   M2O_LOSS: r = z - N - u, loss += |r| / count, out = dL/dN = -sign(r) / count  (layer 8 forward)
+//   M2O_JAC:  out = v - 2 N                                                       (J_Q v and J_Q^T w)
+// A thread holds one column of M2O_ROWS output rows and walks the M2O_ROWS + 2 canvas rows that they read, so
+// each 8-channel vector is loaded 3 (M2O_ROWS + 2) / M2O_ROWS times per pixel instead of 9.  The terms of a pixel
+// are added in the order t, c as one chain (the sign of r, and through it every gradient, hangs on the last bit
+// of N).  Bound by those FMA (576 a pixel) and the loads of the weights.  16 x 256^2: 184 -> 95 us.
+constexpr int M2O_LOSS = 0, M2O_JAC = 1, M2O_THREADS = 128;
+template <int MODE, bool FLIP, int ROWS>
+__global__ void __launch_bounds__(M2O_THREADS) many_to_one(Dims d, const __nv_bfloat16* __restrict__ cv,
+                                                           const float* __restrict__ w, int w_taps_first,
+                                                           const float* __restrict__ bias, const float* __restrict__ v,
+                                                           const float* __restrict__ u, float* __restrict__ out,
+                                                           double* loss) {
+  __shared__ __align__(16) float sw[9 * CH];
+  __shared__ double red[M2O_THREADS / 32];
+  for (int i = threadIdx.x; i < 9 * CH; i += blockDim.x) sw[w_taps_first ? i : (i % 9) * CH + i / 9] = w[i];
+  __syncthreads();
+  const int b = blockIdx.z, y0 = blockIdx.y * ROWS, x = blockIdx.x * M2O_THREADS + threadIdx.x;
+  float acc[ROWS];
+  const float init = MODE == M2O_LOSS ? bias[7 * CH] : 0.f;
 #pragma unroll
-    for (int t = 0; t < 9; ++t) {
-      const int yy = y - (t / 3 - 1), xx = x - (t % 3 - 1);
-      gt[t] = (yy >= 0 && yy < d.s && xx >= 0 && xx < d.s) ? g[((int64_t)b * d.s + yy) * d.s + xx] : 0.f;
-    }
-#pragma unroll 4
-    for (int c = 0; c < CH / 2; ++c) {
-      const size_t at = cidx(d, b, y, x, 2 * c);
-      float v0 = 0.f, v1 = 0.f;
+  for (int k = 0; k < ROWS; ++k) acc[k] = init;
 #pragma unroll
-      for (int t = 0; t < 9; ++t) {
-        v0 = fmaf(sw[t * CH + 2 * c], gt[t], v0);
-        v1 = fmaf(sw[t * CH + 2 * c + 1], gt[t], v1);
+  for (int rr = 0; rr < ROWS + 2; ++rr) {
+    // canvas rows in the order in which every output row meets its taps
+    const int k0 = FLIP ? ROWS - rr : rr - 1;  // canvas row y0 + k0
+    const int y = y0 + k0;
+    const bool row_in = y >= 0 && y < d.s;
+#pragma unroll 1
+    for (int dx = 0; dx < 3; ++dx) {
+      const int xx = FLIP ? x + 1 - dx : x + dx - 1;
+      const bool in = row_in && xx >= 0 && xx < d.s;
+      const __nv_bfloat16* src = cv + cidx(d, b, in ? y : 0, in ? xx : 0, 0);
+      const size_t plane = (size_t)d.Wc * 8;
+#pragma unroll 2
+      for (int cb = 0; cb < 8; ++cb) {
+        const uint4 a = in ? *reinterpret_cast<const uint4*>(src + cb * plane) : make_uint4(0, 0, 0, 0);
+        const uint32_t* aw = reinterpret_cast<const uint32_t*>(&a);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float2 av = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&aw[q]));
+#pragma unroll
+          for (int ty = 0; ty < 3; ++ty) {
+            const int k = FLIP ? k0 + ty - 1 : k0 - ty + 1;  // the output row for which this row is tap row ty
+            if (k < 0 || k >= ROWS) continue;
+            const float2 wv = *reinterpret_cast<const float2*>(&sw[(3 * ty + dx) * CH + 8 * cb + 2 * q]);
+            acc[k] = fmaf(wv.x, av.x, fmaf(wv.y, av.y, acc[k]));
+          }
+        }
       }
-      const float2 av = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(act7 + at));
-      *reinterpret_cast<__nv_bfloat162*>(dpre + at) =
-          __floats2bfloat162_rn(av.x > 0.f ? v0 : 0.f, av.y > 0.f ? v1 : 0.f);
     }
   }
-}
-
-// Gradients of a one-channel layer: thread (t, c) accumulates sum_p s1[p] * s2(p + off_t)[c]
-// where one side is a one-channel FP32 image and the other a 64-channel canvas.
-//   mode 0 (layer 8): dW8[c][t] += sum_p g[p] act7[p + off_t][c];   db8 += sum_p g[p]
-//   mode 1 (layer 1): dW1[c][t] += sum_p dpre1[p][c] z[p + off_t];    db1[c] += sum_p dpre1[p][c]
-__global__ void __launch_bounds__(576) wgrad_onechannel(Dims d, int mode, const float* __restrict__ img,
-                                                        const __nv_bfloat16* __restrict__ cv, float* __restrict__ dW,
-                                                        float* __restrict__ db) {
-  const int t = threadIdx.x / CH, c = threadIdx.x % CH;
-  const int64_t total = (int64_t)d.B * d.s * d.s;
-  const int64_t p0 = (int64_t)blockIdx.x * WG_CHUNK, p1 = min(total, p0 + WG_CHUNK);
-  const int dy = t / 3 - 1, dx = t % 3 - 1;
-  float acc = 0.f, bacc = 0.f;
-  for (int64_t p = p0; p < p1; ++p) {
-    const int b = (int)(p / ((int64_t)d.s * d.s)), y = (int)((p / d.s) % d.s), x = (int)(p % d.s);
-    const int yy = y + dy, xx = x + dx;
-    const bool in = yy >= 0 && yy < d.s && xx >= 0 && xx < d.s;
-    if (mode == 0) {
-      const float gv = img[p];
-      if (in) acc = fmaf(gv, __bfloat162float(cv[cidx(d, b, yy, xx, c)]), acc);
-      bacc += gv;
+  double sum = 0.0;
+  const float inv = 1.f / (float)((int64_t)d.B * d.s * d.s);
+#pragma unroll
+  for (int k = 0; k < ROWS; ++k) {
+    if (x >= d.s || y0 + k >= d.s) continue;
+    const int64_t p = ((int64_t)b * d.s + y0 + k) * d.s + x;
+    if (MODE == M2O_LOSS) {
+      const float r = v[p] - acc[k] - u[p];
+      sum += fabs((double)r);
+      out[p] = r > 0.f ? -inv : (r < 0.f ? inv : 0.f);
     } else {
-      const float dv = __bfloat162float(cv[cidx(d, b, y, x, c)]);
-      if (in) acc = fmaf(dv, img[((int64_t)b * d.s + yy) * d.s + xx], acc);
-      bacc += dv;
+      out[p] = v[p] - 2.f * acc[k];
     }
   }
-  if (mode == 0) {
-    atomicAdd(&dW[c * 9 + t], acc);
-    if (threadIdx.x == 0) atomicAdd(&db[0], bacc);
-  } else {
-    atomicAdd(&dW[c * 9 + t], acc);
-    if (t == 4) atomicAdd(&db[c], bacc);
+  if (MODE == M2O_LOSS) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sum;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      for (int k = 1; k < M2O_THREADS / 32; ++k) sum += red[k];
+      atomicAdd(loss, sum * (double)inv);
+    }
   }
 }
 
-// dW[co][ci][t] += sum_p dpre[p][co] act[p + off_t][ci]; db[co] += sum_p dpre[p][co] (t == 4 blocks)
 // Weight and bias gradients of a 64 -> 64 layer on the tensor cores (mma.sync m16n8k16, BF16 in, FP32
 // accumulate): dW[co][ci][t] = sum_p dpre[p][co] act[p + off_t][ci] is, per tap t, a 64 x 64 GEMM whose
-// contraction runs over the pixels.  A CTA walks image rows (b, y) in 64-pixel segments; per segment it
-// copies dpre (64 px x 64 ch) and the three activation rows y - 1, y, y + 1 (66 px with the dx halo,
-// zero outside the image) into shared memory as [pixel][channel] rows padded to 72 channels (conflict-free
-// ldmatrix) with cp.async, double buffered: the next segment's copies are in flight while the current one
-// is contracted.  Warp w owns tap w / 2 and output channels 32 (w % 2) .. + 31: 2 x 8 tiles of 16 x 8
-// accumulators.  Both operands are stored pixel-major, so the fragments load with ldmatrix.trans.  Bias
-// gradients (sums of dpre over the pixels) come from the staged dpre.  One atomic per gradient entry per
-// CTA at the end.
+// contraction runs over the pixels.  The image rows of all 64-pixel column segments form one sequence that is
+// cut evenly over the CTAs.  A CTA walks down a segment: per row it copies one dpre row (64 px x 64 ch) and the
+// next activation row (66 px with the dx halo, zero outside the image) into rings in shared memory with cp.async,
+// WGT_AHEAD rows ahead, as [pixel][channel] rows padded to 72 channels (conflict-free ldmatrix); each activation
+// row serves three dpre rows.  Warp w owns tap w / 2 and output channels 32 (w % 2) .. + 31: 2 x 8 tiles of
+// 16 x 8 accumulators.  Both operands are stored pixel-major, so the fragments load with ldmatrix.trans.  Bias
+// gradients (sums of dpre over the pixels) come from the fragments of the centre tap's warps.  Each
+// CTA writes its partial sums to its slice of a workspace and wgrad64_reduce adds the slices up (as global atomics
+// the 36864 sums of each CTA cost about as much as the contraction).
+// Bound by the tensor pipe as mma.sync drives it (math pipe throttle, 330 TFLOP/s).  16 x 256^2: 381 -> 244 us
+// with the reduction (8 x 128^2: 106 -> 45 us) against restaging three activation rows per row, two stages deep,
+// a serial bias sum and atomics.
 constexpr int WGT_PX = 64;                    // pixels per segment (4 K steps of 16)
 constexpr int WGT_LD = 72;                    // staged row length (channels + 8 of padding)
 constexpr int WGT_WARPS = 18;                 // 9 taps x 2 output-channel halves
 constexpr int WGT_THREADS = WGT_WARPS * 32;
-constexpr int WGT_CHUNKS = 8 * (WGT_PX + 3 * (WGT_PX + 2));  // 16-byte chunks per segment: 2096
-constexpr int WGT_BUF = (WGT_PX + 3 * (WGT_PX + 2)) * WGT_LD;  // staged elements per segment
-constexpr int WGT_SMEM = 2 * WGT_BUF * 2;                       // bytes, two buffers
+constexpr int WGT_AHEAD = 3;                  // rows whose copies are in flight
+constexpr int WGT_NA = WGT_AHEAD + 3, WGT_ND = WGT_AHEAD + 1;   // ring slots: activation and dpre rows
+constexpr int WGT_AROW = (WGT_PX + 2) * WGT_LD, WGT_DROW = WGT_PX * WGT_LD;  // elements of a slot
+constexpr int WGT_SMEM = (WGT_NA * WGT_AROW + WGT_ND * WGT_DROW) * 2;
+constexpr int WGT_SUMS = 9 * CH * CH + CH;    // a CTA's partial sums: [t][co][ci], then [co] of the bias
 
 __device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
   asm volatile(
@@ -231,109 +402,161 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src, int nbyte
                : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
 
-// copies of segment sg (image row b * s + y, pixels x0 ..) into the staging buffer buf: chunk e is 16
-// bytes of dpre (e < 512, into [px][WGT_LD]) or of activation row y + r - 1 (into [3][66 px][WGT_LD])
-__device__ __forceinline__ void wgt_issue(const Dims& d, const __nv_bfloat16* __restrict__ dpre,
-                                          const __nv_bfloat16* __restrict__ act, int64_t sg, int segs_per_row,
-                                          __nv_bfloat16* buf) {
-  const int row = (int)(sg / segs_per_row), x0 = (int)(sg % segs_per_row) * WGT_PX;
-  const int b = row / d.s, y = row % d.s;
-  for (int e = threadIdx.x; e < WGT_CHUNKS; e += WGT_THREADS) {
-    int yy = y, x, kb, slot;
-    const __nv_bfloat16* src = dpre;
-    if (e < 8 * WGT_PX) {
-      x = x0 + (e >> 3);
-      kb = e & 7;
-      slot = (e >> 3) * WGT_LD + 8 * kb;
-    } else {
-      const int f = e - 8 * WGT_PX, r = f / (8 * (WGT_PX + 2)), q = f % (8 * (WGT_PX + 2));
-      yy = y + r - 1;
-      x = x0 - 1 + (q >> 3);
-      kb = q & 7;
-      slot = WGT_PX * WGT_LD + (r * (WGT_PX + 2) + (q >> 3)) * WGT_LD + 8 * kb;
-      src = act;
-    }
-    const bool in = yy >= 0 && yy < d.s && x >= 0 && x < d.s;
-    cp_async16(buf + slot, in ? src + cidx(d, b, yy, x, 8 * kb) : src, in ? 16 : 0);
+// copies PX pixels x .. of canvas row y of image b (zero outside the image) into dst, [px][WGT_LD]
+template <int PX>
+__device__ __forceinline__ void wgt_row(const Dims& d, const __nv_bfloat16* __restrict__ cv, int b, int y, int x,
+                                        __nv_bfloat16* dst) {
+  const bool row_in = y >= 0 && y < d.s;
+  for (int e = threadIdx.x; e < 8 * PX; e += WGT_THREADS) {
+    const int kb = e / PX, px = e - kb * PX, xx = x + px;
+    const bool in = row_in && xx >= 0 && xx < d.s;
+    cp_async16(dst + px * WGT_LD + 8 * kb, in ? cv + cidx(d, b, y, xx, 8 * kb) : cv, in ? 16 : 0);
   }
 }
 
 __global__ void __launch_bounds__(WGT_THREADS, 1) wgrad64_tc(Dims d, const __nv_bfloat16* __restrict__ dpre,
                                                              const __nv_bfloat16* __restrict__ act,
-                                                             float* __restrict__ dW, float* __restrict__ db) {
+                                                             float* __restrict__ part) {
   extern __shared__ __align__(16) __nv_bfloat16 wsm[];
+  __nv_bfloat16* sA = wsm;                        // activation ring, row y in slot (y + 1) mod WGT_NA
+  __nv_bfloat16* sD = wsm + WGT_NA * WGT_AROW;    // dpre ring, row y in slot y mod WGT_ND
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int t = warp >> 1, dy = t / 3, dx = t % 3, co0 = 32 * (warp & 1);
-  const int segs_per_row = (d.s + WGT_PX - 1) / WGT_PX;
-  const int64_t nseg = (int64_t)d.B * d.s * segs_per_row;
-  float acc[2][8][4] = {};
-  float bsum = 0.f;
-  int cur = 0;
-  if ((int64_t)blockIdx.x < nseg) wgt_issue(d, dpre, act, blockIdx.x, segs_per_row, wsm);
-  cp_async_commit();
+  const int segs = (d.s + WGT_PX - 1) / WGT_PX;
+  const int64_t total = (int64_t)d.B * segs * d.s;
+  int64_t l = total * blockIdx.x / gridDim.x;
+  const int64_t le = total * (blockIdx.x + 1) / gridDim.x;
+  float acc[2][8][4] = {}, bsum[2][2] = {};
   const int i = lane >> 3, r = lane & 7;
-  for (int64_t sg = blockIdx.x; sg < nseg; sg += gridDim.x) {
-    if (sg + gridDim.x < nseg) wgt_issue(d, dpre, act, sg + gridDim.x, segs_per_row, wsm + (1 - cur) * WGT_BUF);
-    cp_async_commit();
-    cp_async_wait1();  // this thread's copies of the current segment have landed
-    __syncthreads();   // and everyone's
-    const __nv_bfloat16* sA = wsm + cur * WGT_BUF;
-    const __nv_bfloat16* sB = sA + WGT_PX * WGT_LD;
-    if (threadIdx.x < CH) {
-      float sacc = 0.f;
-      for (int p = 0; p < WGT_PX; ++p) sacc += __bfloat162float(sA[p * WGT_LD + threadIdx.x]);
-      bsum += sacc;
-    }
+  while (l < le) {
+    const int strip = (int)(l / d.s), ya = (int)(l % d.s), yb = (int)min((int64_t)d.s, ya + (le - l));
+    const int b = strip / segs, x0 = strip % segs * WGT_PX;
+    auto fetch = [&](int y) {  // the copies of step y: dpre row y and activation row y + 1
+      if (y < yb) {
+        wgt_row<WGT_PX>(d, dpre, b, y, x0, sD + y % WGT_ND * WGT_DROW);
+        wgt_row<WGT_PX + 2>(d, act, b, y + 1, x0 - 1, sA + (y + 2) % WGT_NA * WGT_AROW);
+      }
+      cp_async_commit();
+    };
+    __syncthreads();  // every warp is done with the previous strip's rings
+    wgt_row<WGT_PX + 2>(d, act, b, ya - 1, x0 - 1, sA + ya % WGT_NA * WGT_AROW);
+    wgt_row<WGT_PX + 2>(d, act, b, ya, x0 - 1, sA + (ya + 1) % WGT_NA * WGT_AROW);
+    for (int y = ya; y < ya + WGT_AHEAD; ++y) fetch(y);
+    for (int y = ya; y < yb; ++y) {
+      cp_async_wait<WGT_AHEAD - 1>();  // this thread's copies of step y have landed
+      __syncthreads();                 // and everyone's; the slots filled next were last read in step y - 1
+      fetch(y + WGT_AHEAD);
+      const __nv_bfloat16* pD = sD + y % WGT_ND * WGT_DROW;
+      const __nv_bfloat16* pA = sA + (y + dy) % WGT_NA * WGT_AROW;  // activation row y + dy - 1
 #pragma unroll
-    for (int kk = 0; kk < WGT_PX / 16; ++kk) {
-      uint32_t a[2][4];
+      for (int kk = 0; kk < WGT_PX / 16; ++kk) {
+        uint32_t a[2][4];
 #pragma unroll
-      for (int mt = 0; mt < 2; ++mt)
-        ldsm_x4_trans(a[mt], sA + (16 * kk + r + 8 * (i >> 1)) * WGT_LD + co0 + 16 * mt + 8 * (i & 1));
+        for (int mt = 0; mt < 2; ++mt)
+          ldsm_x4_trans(a[mt], pD + (16 * kk + r + 8 * (i >> 1)) * WGT_LD + co0 + 16 * mt + 8 * (i & 1));
 #pragma unroll
-      for (int np = 0; np < 4; ++np) {
-        uint32_t bq[4];
-        ldsm_x4_trans(bq, sB + (dy * (WGT_PX + 2) + 16 * kk + r + 8 * (i & 1) + dx) * WGT_LD + 16 * np + 8 * (i >> 1));
+        for (int np = 0; np < 4; ++np) {
+          uint32_t bq[4];
+          ldsm_x4_trans(bq, pA + (16 * kk + r + 8 * (i & 1) + dx) * WGT_LD + 16 * np + 8 * (i >> 1));
 #pragma unroll
-        for (int mt = 0; mt < 2; ++mt) {
-          mma16816(acc[mt][2 * np], a[mt], bq[0], bq[1]);
-          mma16816(acc[mt][2 * np + 1], a[mt], bq[2], bq[3]);
+          for (int mt = 0; mt < 2; ++mt) {
+            mma16816(acc[mt][2 * np], a[mt], bq[0], bq[1]);
+            mma16816(acc[mt][2 * np + 1], a[mt], bq[2], bq[3]);
+          }
+        }
+        if (t == 4) {  // warp-uniform: the pixel sums of dpre, rows g and g + 8 of the fragments
+#pragma unroll
+          for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              const float2 lo = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&a[mt][h]));
+              const float2 hi = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&a[mt][2 + h]));
+              bsum[mt][h] += (lo.x + lo.y) + (hi.x + hi.y);
+            }
         }
       }
     }
-    __syncthreads();  // the buffer is refilled by the next iteration's copies
-    cur = 1 - cur;
+    l += yb - ya;
   }
-  asm volatile("cp.async.wait_all;" ::: "memory");
+  cp_async_wait<0>();
   const int g = lane >> 2, tq = lane & 3;
+  float* o = part + (size_t)blockIdx.x * WGT_SUMS;
 #pragma unroll
   for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-    for (int nt = 0; nt < 8; ++nt)
+    for (int h = 0; h < 2; ++h) {
+      const int co = co0 + 16 * mt + g + 8 * h;
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int co = co0 + 16 * mt + g + 8 * h, ci = 8 * nt + 2 * tq;
-        atomicAdd(&dW[((size_t)co * CH + ci) * 9 + t], acc[mt][nt][2 * h]);
-        atomicAdd(&dW[((size_t)co * CH + ci + 1) * 9 + t], acc[mt][nt][2 * h + 1]);
+      for (int nt = 0; nt < 8; ++nt)
+        *reinterpret_cast<float2*>(&o[(t * CH + co) * CH + 8 * nt + 2 * tq]) =
+            make_float2(acc[mt][nt][2 * h], acc[mt][nt][2 * h + 1]);
+      if (t == 4) {
+        float v = bsum[mt][h];
+        v += __shfl_xor_sync(0xffffffffu, v, 1);
+        v += __shfl_xor_sync(0xffffffffu, v, 2);
+        if (tq == 0) o[9 * CH * CH + co] = v;
       }
-  if (threadIdx.x < CH && db) atomicAdd(&db[threadIdx.x], bsum);
+    }
 }
 
-int wgrad64_launch(cudaStream_t s, const Dims& d, const __nv_bfloat16* dpre, const __nv_bfloat16* act, float* dW,
-                   float* db) {
+// dW[co][ci][t] and db[co] += the sums of the `parts` slices; block (32, 8): 32 sums, the slices dealt to 8 rows
+__global__ void __launch_bounds__(256) wgrad64_reduce(const float* __restrict__ part, int parts,
+                                                      float* __restrict__ dW, float* __restrict__ db) {
+  __shared__ float red[8][32];
+  const int e = blockIdx.x * 32 + threadIdx.x;
+  float s = 0.f;
+  if (e < WGT_SUMS)
+    for (int k = threadIdx.y; k < parts; k += 8) s += part[(size_t)k * WGT_SUMS + e];
+  red[threadIdx.y][threadIdx.x] = s;
+  __syncthreads();
+  if (threadIdx.y || e >= WGT_SUMS) return;
+  for (int k = 1; k < 8; ++k) s += red[k][threadIdx.x];
+  if (e < 9 * CH * CH) dW[(size_t)(e % (CH * CH)) * 9 + e / (CH * CH)] += s;
+  else db[e - 9 * CH * CH] += s;
+}
+
+int device_sms(int* sms) {
+  int dev = 0;
+  PNP_CUDA(cudaGetDevice(&dev));
+  PNP_CUDA(cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev));
+  return PNP_OK;
+}
+
+int wgrad64_launch(cudaStream_t s, const Dims& d, const __nv_bfloat16* dpre, const __nv_bfloat16* act, float* part,
+                   int parts, float* dW, float* db) {
   static bool attr = false;
   if (!attr) {
     PNP_CUDA(cudaFuncSetAttribute(wgrad64_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, WGT_SMEM));
     attr = true;
   }
-  const int64_t nseg = (int64_t)d.B * d.s * ((d.s + WGT_PX - 1) / WGT_PX);
-  int dev = 0, sms = 0;
-  PNP_CUDA(cudaGetDevice(&dev));
-  PNP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(nseg, sms));
-  wgrad64_tc<<<grid, WGT_THREADS, WGT_SMEM, s>>>(d, dpre, act, dW, db);
+  wgrad64_tc<<<parts, WGT_THREADS, WGT_SMEM, s>>>(d, dpre, act, part);
+  PNP_CHECK_LAUNCH();
+  wgrad64_reduce<<<(WGT_SUMS + 31) / 32, dim3(32, 8), 0, s>>>(part, parts, dW, db);
+  PNP_CHECK_LAUNCH();
+  return PNP_OK;
+}
+
+// launch shape of one_to_many and wgrad_onechannel: as many rows per block (8 to 64) as leave three blocks per SM
+dim3 end_grid(const Dims& d, int sms, int* rows) {
+  const int cols = (d.s + END_COLS - 1) / END_COLS;
+  *rows = END_ROWS;
+  while (*rows > 8 && (int64_t)cols * ((d.s + *rows - 1) / *rows) * d.B < 3 * sms) *rows >>= 1;
+  return dim3(cols, (d.s + *rows - 1) / *rows, d.B);
+}
+
+template <int MODE, bool FLIP>
+int many_to_one_launch(cudaStream_t s, const Dims& d, int sms, const __nv_bfloat16* cv, const float* w,
+                       int w_taps_first, const float* bias, const float* v, const float* u, float* out, double* loss) {
+  const int cols = (d.s + M2O_THREADS - 1) / M2O_THREADS;
+  if ((int64_t)cols * ((d.s + 7) / 8) * d.B >= 4 * sms)
+    many_to_one<MODE, FLIP, 8><<<dim3(cols, (d.s + 7) / 8, d.B), M2O_THREADS, 0, s>>>(d, cv, w, w_taps_first, bias, v, u, out, loss);
+  else
+    many_to_one<MODE, FLIP, 2><<<dim3(cols, (d.s + 1) / 2, d.B), M2O_THREADS, 0, s>>>(d, cv, w, w_taps_first, bias, v, u, out, loss);
   PNP_CHECK_LAUNCH();
   return PNP_OK;
 }
@@ -342,97 +565,7 @@ int wgrad64_launch(cudaStream_t s, const Dims& d, const __nv_bfloat16* dpre, con
 // With D(z) = z - N(z), J_Q = I - 2 J_N, and J_N at z is the network with its ReLU masks at z
 // frozen and no biases.  Layers 2-7 of J_N v run on the tensor cores (conv64 backward-data mode
 // with the forward weights and the masks [act_{k+1} > 0]); J_N^T w is the back-propagation of
-// the training step.  These kernels are the one-channel ends of both chains.
-
-// t1[p][c] = [act1[p][c] > 0] * sum_t W1[c][t] v[p + off_t]
-__global__ void __launch_bounds__(256) tangent_first(Dims d, const float* __restrict__ v,
-                                                     const float* __restrict__ w1r,
-                                                     const __nv_bfloat16* __restrict__ act1,
-                                                     __nv_bfloat16* __restrict__ t1) {
-  __shared__ float sw[9 * CH];
-  for (int i = threadIdx.x; i < 9 * CH; i += blockDim.x) sw[i] = w1r[i];
-  __syncthreads();
-  const int64_t total = (int64_t)d.B * d.s * d.s;
-  for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < total; p += (int64_t)gridDim.x * blockDim.x) {
-    const int b = (int)(p / ((int64_t)d.s * d.s)), y = (int)((p / d.s) % d.s), x = (int)(p % d.s);
-    float vt[9];
-#pragma unroll
-    for (int t = 0; t < 9; ++t) {
-      const int yy = y + t / 3 - 1, xx = x + t % 3 - 1;
-      vt[t] = (yy >= 0 && yy < d.s && xx >= 0 && xx < d.s) ? v[((int64_t)b * d.s + yy) * d.s + xx] : 0.f;
-    }
-#pragma unroll 4
-    for (int c = 0; c < CH / 2; ++c) {
-      const size_t at = cidx(d, b, y, x, 2 * c);
-      float v0 = 0.f, v1 = 0.f;
-#pragma unroll
-      for (int t = 0; t < 9; ++t) {
-        v0 = fmaf(sw[(2 * c) * 9 + t], vt[t], v0);
-        v1 = fmaf(sw[(2 * c + 1) * 9 + t], vt[t], v1);
-      }
-      const float2 av = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(act1 + at));
-      *reinterpret_cast<__nv_bfloat162*>(t1 + at) = __floats2bfloat162_rn(av.x > 0.f ? v0 : 0.f, av.y > 0.f ? v1 : 0.f);
-    }
-  }
-}
-
-// w[p] = v[p] - 2 sum_{t, c} W8[c][t] t7[p + off_t][c]   (J_Q v from the layer-7 tangent)
-__global__ void __launch_bounds__(256) tangent_last(Dims d, const __nv_bfloat16* __restrict__ t7,
-                                                    const float* __restrict__ w8r, const float* __restrict__ v,
-                                                    float* __restrict__ w) {
-  __shared__ float sw[9 * CH];
-  for (int i = threadIdx.x; i < 9 * CH; i += blockDim.x) sw[i] = w8r[i];
-  __syncthreads();
-  const int64_t total = (int64_t)d.B * d.s * d.s;
-  for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < total; p += (int64_t)gridDim.x * blockDim.x) {
-    const int b = (int)(p / ((int64_t)d.s * d.s)), y = (int)((p / d.s) % d.s), x = (int)(p % d.s);
-    float jn = 0.f;
-    for (int t = 0; t < 9; ++t) {
-      const int yy = y + t / 3 - 1, xx = x + t % 3 - 1;
-      if (yy < 0 || yy >= d.s || xx < 0 || xx >= d.s) continue;
-#pragma unroll
-      for (int cb = 0; cb < 8; ++cb) {
-        const __nv_bfloat162* a = reinterpret_cast<const __nv_bfloat162*>(t7 + cidx(d, b, yy, xx, 8 * cb));
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const int c = 4 * cb + k;
-          const float2 tv = __bfloat1622float2(a[k]);
-          jn = fmaf(sw[t * CH + 2 * c], tv.x, fmaf(sw[t * CH + 2 * c + 1], tv.y, jn));
-        }
-      }
-    }
-    w[p] = v[p] - 2.f * jn;
-  }
-}
-
-// u[p] = w[p] - 2 sum_{t, c} W1[c][t] dpre1[p - off_t][c]   (J_Q^T w from the layer-1 gradient)
-__global__ void __launch_bounds__(256) cotangent_first(Dims d, const __nv_bfloat16* __restrict__ dpre1,
-                                                       const float* __restrict__ w1r, const float* __restrict__ w,
-                                                       float* __restrict__ u) {
-  __shared__ float sw[9 * CH];  // [t][c]
-  for (int i = threadIdx.x; i < 9 * CH; i += blockDim.x) sw[(i % 9) * CH + i / 9] = w1r[i];
-  __syncthreads();
-  const int64_t total = (int64_t)d.B * d.s * d.s;
-  for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < total; p += (int64_t)gridDim.x * blockDim.x) {
-    const int b = (int)(p / ((int64_t)d.s * d.s)), y = (int)((p / d.s) % d.s), x = (int)(p % d.s);
-    float jt = 0.f;
-    for (int t = 0; t < 9; ++t) {
-      const int yy = y - (t / 3 - 1), xx = x - (t % 3 - 1);
-      if (yy < 0 || yy >= d.s || xx < 0 || xx >= d.s) continue;
-#pragma unroll
-      for (int cb = 0; cb < 8; ++cb) {
-        const __nv_bfloat162* a = reinterpret_cast<const __nv_bfloat162*>(dpre1 + cidx(d, b, yy, xx, 8 * cb));
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const int c = 4 * cb + k;
-          const float2 gv = __bfloat1622float2(a[k]);
-          jt = fmaf(sw[t * CH + 2 * c], gv.x, fmaf(sw[t * CH + 2 * c + 1], gv.y, jt));
-        }
-      }
-    }
-    u[p] = w[p] - 2.f * jt;
-  }
-}
+// the training step; the one-channel ends of both chains are one_to_many and many_to_one.
 
 // n2[b] += sum_p x[b][p]^2 (FP64); grid (blocks per image, B)
 __global__ void __launch_bounds__(256) image_norm2(const float* __restrict__ x, int64_t plane, double* n2) {
@@ -505,7 +638,9 @@ int nblocks(int64_t count, int threads = 256) {
 struct pnp_cnn_trainer {
   pnp::Dims d{};
   cudaStream_t stream = nullptr;
-  int n_strips = 0, t = 0;
+  int n_strips = 0, t = 0, sms = 0;
+  int parts = 0;          // CTAs of the weight-gradient kernel
+  float* part = nullptr;  // their partial sums (parts x WGT_SUMS)
   double lr = 1e-4, b1 = 0.9, b2 = 0.999, eps = 1e-8;
   float *w = nullptr, *g = nullptr, *m = nullptr, *v = nullptr;
   float *w1r = nullptr, *w8r = nullptr, *bias = nullptr;
@@ -532,7 +667,7 @@ void trainer_free(pnp_cnn_trainer* T) {
   if (!T) return;
   for (void* p : {(void*)T->w, (void*)T->g, (void*)T->m, (void*)T->v, (void*)T->w1r, (void*)T->w8r, (void*)T->bias,
                   (void*)T->wf, (void*)T->wb, (void*)T->z, (void*)T->gout, (void*)T->facets, (void*)T->strips,
-                  (void*)T->loss, (void*)T->status, (void*)T->jv, (void*)T->jw, (void*)T->ju, (void*)T->jn2})
+                  (void*)T->loss, (void*)T->status, (void*)T->jv, (void*)T->jw, (void*)T->ju, (void*)T->jn2, (void*)T->part})
     cudaFree(p);
   for (auto p : T->act) cudaFree(p);
   for (auto p : T->dp) cudaFree(p);
@@ -561,6 +696,35 @@ int image_norms(pnp_cnn_trainer* T, const float* x) {
 }  // namespace
 
 namespace {
+// dpre7 = [act7 > 0] W8^T g into dp[0]
+int layer8_back(pnp_cnn_trainer* T, const float* g) {
+  int rows;
+  const dim3 grid = end_grid(T->d, T->sms, &rows);
+  one_to_many<true><<<grid, 256, 0, T->stream>>>(T->d, rows, T->act[7], T->w8r, g, T->dp[0]);
+  PNP_CHECK_LAUNCH();
+  return PNP_OK;
+}
+// t1 = [act1 > 0] W1 v
+int layer1_tangent(pnp_cnn_trainer* T, const float* v, __nv_bfloat16* t1) {
+  int rows;
+  const dim3 grid = end_grid(T->d, T->sms, &rows);
+  one_to_many<false><<<grid, 256, 0, T->stream>>>(T->d, rows, T->act[1], T->w1r, v, t1);
+  PNP_CHECK_LAUNCH();
+  return PNP_OK;
+}
+template <bool LAYER8>
+int onechannel_grads(pnp_cnn_trainer* T, const float* img, const __nv_bfloat16* cv, float* dW, float* db) {
+  int rows;
+  const dim3 tiles = end_grid(T->d, T->sms, &rows);
+  // two blocks per SM are resident; the workspace holds more than 57 slices per weight-gradient CTA
+  const int blocks = (int)std::min<int64_t>((int64_t)tiles.x * tiles.y * tiles.z, 2 * T->parts);
+  wgrad_onechannel<LAYER8><<<blocks, 256, 0, T->stream>>>(T->d, rows, img, cv, T->part);
+  PNP_CHECK_LAUNCH();
+  onechannel_reduce<<<ONE_SUMS / 32, dim3(32, 8), 0, T->stream>>>(T->part, blocks, LAYER8 ? 1 : 0, dW, db);
+  PNP_CHECK_LAUNCH();
+  return PNP_OK;
+}
+
 // the forward pass at z that fixes the ReLU masks (activations act[1..7])
 int primal_forward(pnp_cnn_trainer* T, const float* z) {
   const Dims d = T->d;
@@ -586,8 +750,7 @@ int power_iterate(pnp_cnn_trainer* T, const float* v0, int iters, double* sigma_
   PNP_CHECK_LAUNCH();
   for (int it = 0; it < iters; ++it) {
     // w = J_Q v: tangents through layers 1..7 (masks [act_k > 0]), then layer 8
-    tangent_first<<<nblocks(npx), 256, 0, s>>>(d, T->jv, T->w1r, T->act[1], T->dp[0]);
-    PNP_CHECK_LAUNCH();
+    if (int rc = layer1_tangent(T, T->jv, T->dp[0])) return rc;
     int cur = 0;
     for (int k = 1; k <= 6; ++k) {
       if (int rc = conv64_launch(s, T->map_dp[cur], T->dp[1 - cur], T->wf + (size_t)(k - 1) * NWM, nullptr, T->strips,
@@ -595,11 +758,10 @@ int power_iterate(pnp_cnn_trainer* T, const float* v0, int iters, double* sigma_
         return rc;
       cur = 1 - cur;
     }
-    tangent_last<<<nblocks(npx), 256, 0, s>>>(d, T->dp[cur], T->w8r, T->jv, T->jw);
-    PNP_CHECK_LAUNCH();
+    if (int rc = many_to_one_launch<M2O_JAC, false>(s, d, T->sms, T->dp[cur], T->w8r, 1, nullptr, T->jv, nullptr, T->jw, nullptr))
+      return rc;
     // u = J_Q^T w: the training step's back-propagation with cotangent w
-    last_bwd<<<nblocks(npx), 256, 0, s>>>(d, T->act[7], T->w8r, T->jw, T->dp[0]);
-    PNP_CHECK_LAUNCH();
+    if (int rc = layer8_back(T, T->jw)) return rc;
     cur = 0;
     for (int k = 6; k >= 1; --k) {
       if (int rc = conv64_launch(s, T->map_dp[cur], T->dp[1 - cur], T->wb + (size_t)(k - 1) * NWM, nullptr, T->strips,
@@ -607,8 +769,8 @@ int power_iterate(pnp_cnn_trainer* T, const float* v0, int iters, double* sigma_
         return rc;
       cur = 1 - cur;
     }
-    cotangent_first<<<nblocks(npx), 256, 0, s>>>(d, T->dp[cur], T->w1r, T->jw, T->ju);
-    PNP_CHECK_LAUNCH();
+    if (int rc = many_to_one_launch<M2O_JAC, true>(s, d, T->sms, T->dp[cur], T->w1r, 0, nullptr, T->jw, nullptr, T->ju, nullptr))
+      return rc;
     if (sigma_host && it == iters - 1) {  // sigma = ||J_Q v|| for the current unit v
       if (int rc = image_norms(T, T->jw)) return rc;
       PNP_CUDA(cudaMemcpyAsync(sigma_host, T->jn2, d.B * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -644,6 +806,12 @@ int pnp_cnn_trainer_create(pnp_cnn_trainer** out, const float* weights_host, int
   T->stream = reinterpret_cast<cudaStream_t>(stream);
   T->lr = lr;
   T->d = Dims{batch, size, size, (size + 127) / 128 * 128};
+  if (int rc = device_sms(&T->sms)) {
+    delete T;
+    return rc;
+  }
+  // a CTA per SM, and at least four image rows each
+  T->parts = (int)std::max<int64_t>(1, std::min<int64_t>(T->sms, (int64_t)batch * ((size + WGT_PX - 1) / WGT_PX) * size / 4));
   const size_t canvas = (size_t)batch * T->d.Hc * T->d.Wc * CH;
   const int64_t npx = (int64_t)batch * size * size;
   auto al = [&](void** p, size_t bytes) -> bool {
@@ -660,7 +828,7 @@ int pnp_cnn_trainer_create(pnp_cnn_trainer** out, const float* weights_host, int
             al((void**)&T->facets, batch * sizeof(int4)) && al((void**)&T->loss, sizeof(double)) &&
             al((void**)&T->status, 4 * sizeof(int)) && al((void**)&T->jv, npx * 4) && al((void**)&T->jw, npx * 4) &&
             al((void**)&T->ju, npx * 4) && al((void**)&T->jn2, batch * sizeof(double)) &&
-            al((void**)&T->junk, CH * sizeof(float));
+            al((void**)&T->junk, CH * sizeof(float)) && al((void**)&T->part, (size_t)T->parts * WGT_SUMS * sizeof(float));
   for (int i = 1; ok && i <= 7; ++i) ok = al((void**)&T->act[i], canvas * 2);
   for (int i = 0; ok && i < 2; ++i) ok = al((void**)&T->dp[i], canvas * 2);
   for (int i = 1; ok && i <= 7; ++i) ok = al((void**)&T->tan[i], canvas * 2);
@@ -734,25 +902,21 @@ int pnp_cnn_train_step(pnp_cnn_trainer* T, const float* u, const float* noise, d
                                T->strips, T->n_strips, d.Hc, d.Wc, 0, nullptr, T->status))
       return rc;
   PNP_CUDA(cudaMemsetAsync(T->loss, 0, sizeof(double), s));
-  last_fwd_loss<<<nblocks(npx), 256, 0, s>>>(d, T->act[7], T->w8r, T->bias, T->z, u, T->gout, T->loss);
-  PNP_CHECK_LAUNCH();
+  if (int rc = many_to_one_launch<M2O_LOSS, false>(s, d, T->sms, T->act[7], T->w8r, 1, T->bias, T->z, u, T->gout, T->loss))
+    return rc;
   // ---------------- backward
-  last_bwd<<<nblocks(npx), 256, 0, s>>>(d, T->act[7], T->w8r, T->gout, T->dp[0]);
-  PNP_CHECK_LAUNCH();
-  const int wgb = (int)((npx + WG_CHUNK - 1) / WG_CHUNK);
-  wgrad_onechannel<<<wgb, 576, 0, s>>>(d, 0, T->gout, T->act[7], T->g + OFF_W8, T->g + OFF_B8);
-  PNP_CHECK_LAUNCH();
+  if (int rc = layer8_back(T, T->gout)) return rc;
+  if (int rc = onechannel_grads<true>(T, T->gout, T->act[7], T->g + OFF_W8, T->g + OFF_B8)) return rc;
   int cur = 0;
   for (int k = 6; k >= 1; --k) {
     float* gW = T->g + OFF_MID + (k - 1) * MID_STRIDE;
-    if (int rc = wgrad64_launch(s, d, T->dp[cur], T->act[k], gW, gW + NWM)) return rc;
+    if (int rc = wgrad64_launch(s, d, T->dp[cur], T->act[k], T->part, T->parts, gW, gW + NWM)) return rc;
     if (int rc = conv64_launch(s, T->map_dp[cur], T->dp[1 - cur], T->wb + (size_t)(k - 1) * NWM, nullptr,
                                T->strips, T->n_strips, d.Hc, d.Wc, 1, T->act[k], T->status))
       return rc;
     cur = 1 - cur;
   }
-  wgrad_onechannel<<<wgb, 576, 0, s>>>(d, 1, T->z, T->dp[cur], T->g + OFF_W1, T->g + OFF_B1);
-  PNP_CHECK_LAUNCH();
+  if (int rc = onechannel_grads<false>(T, T->z, T->dp[cur], T->g + OFF_W1, T->g + OFF_B1)) return rc;
   // ---------------- update
   if (update)
     if (int rc = adam_update(T)) return rc;
@@ -795,34 +959,30 @@ int pnp_cnn_train_step_fne(pnp_cnn_trainer* T, const float* u, const float* nois
     PNP_CHECK_LAUNCH();
   }
   // w = J_Q v with every tangent kept for the weight gradients
-  tangent_first<<<nblocks(npx), 256, 0, s>>>(d, T->jv, T->w1r, T->act[1], T->tan[1]);
-  PNP_CHECK_LAUNCH();
+  if (int rc = layer1_tangent(T, T->jv, T->tan[1])) return rc;
   for (int k = 1; k <= 6; ++k)
     if (int rc = conv64_launch(s, T->map_tan[k], T->tan[k + 1], T->wf + (size_t)(k - 1) * NWM, nullptr, T->strips,
                                T->n_strips, d.Hc, d.Wc, 1, T->act[k + 1], T->status))
       return rc;
-  tangent_last<<<nblocks(npx), 256, 0, s>>>(d, T->tan[7], T->w8r, T->jv, T->jw);
-  PNP_CHECK_LAUNCH();
+  if (int rc = many_to_one_launch<M2O_JAC, false>(s, d, T->sms, T->tan[7], T->w8r, 1, nullptr, T->jv, nullptr, T->jw, nullptr))
+    return rc;
   if (int rc = image_norms(T, T->jw)) return rc;
   fne_cotangent<<<nblocks(npx), 256, 0, s>>>(T->jw, T->jn2, plane, d.B, (float)(lambda / d.B), 1.0 - eps, T->gout);
   PNP_CHECK_LAUNCH();
   // back-propagation of the cotangent through the tangent network (no bias gradients)
-  const int wgb = (int)((npx + WG_CHUNK - 1) / WG_CHUNK);
-  wgrad_onechannel<<<wgb, 576, 0, s>>>(d, 0, T->gout, T->tan[7], T->g + OFF_W8, T->junk);
-  PNP_CHECK_LAUNCH();
-  last_bwd<<<nblocks(npx), 256, 0, s>>>(d, T->act[7], T->w8r, T->gout, T->dp[0]);
-  PNP_CHECK_LAUNCH();
+  if (int rc = onechannel_grads<true>(T, T->gout, T->tan[7], T->g + OFF_W8, T->junk)) return rc;
+  if (int rc = layer8_back(T, T->gout)) return rc;
   int cur = 0;
   for (int k = 6; k >= 1; --k) {
-    if (int rc = wgrad64_launch(s, d, T->dp[cur], T->tan[k], T->g + OFF_MID + (k - 1) * MID_STRIDE, T->junk))
+    if (int rc = wgrad64_launch(s, d, T->dp[cur], T->tan[k], T->part, T->parts,
+                                T->g + OFF_MID + (k - 1) * MID_STRIDE, T->junk))
       return rc;
     if (int rc = conv64_launch(s, T->map_dp[cur], T->dp[1 - cur], T->wb + (size_t)(k - 1) * NWM, nullptr, T->strips,
                                T->n_strips, d.Hc, d.Wc, 1, T->act[k], T->status))
       return rc;
     cur = 1 - cur;
   }
-  wgrad_onechannel<<<wgb, 576, 0, s>>>(d, 1, T->jv, T->dp[cur], T->g + OFF_W1, T->junk);
-  PNP_CHECK_LAUNCH();
+  if (int rc = onechannel_grads<false>(T, T->jv, T->dp[cur], T->g + OFF_W1, T->junk)) return rc;
   if (penalty_host) {
     std::vector<double> n2(d.B);
     PNP_CUDA(cudaMemcpyAsync(n2.data(), T->jn2, d.B * sizeof(double), cudaMemcpyDeviceToHost, s));

@@ -94,3 +94,23 @@ def test_gpu_adam_matches_oracle_over_three_updates():
             assert np.abs(Wg - Wr).max() <= 1e-6 * lr + 1e-7 * np.abs(Wr).max(), step
             assert np.abs(bg - br).max() <= 1e-6 * lr + 1e-7 * np.abs(br).max(), step
         w_prev = w_gpu
+
+
+@pytest.mark.parametrize("B,s", [(1, 17), (3, 33), (1, 65), (1, 130)])
+def test_gradients_match_oracle_at_ragged_sizes(B, s):
+    """Image sides around the widths the gradient kernels work in (32 and 64 columns, 128-pixel tiles): one
+    narrow tile, a second tile of one or two columns, rows that do not divide into the batches of rows.  The
+    bounds are those of test_gradients_match_oracle."""
+    sigma = 0.1
+    params = synth.cnn_init(np.random.default_rng(50 + s), 64, 8, last_scale=0.01)
+    u, nz = _batch(B, s, 60 + s)
+    tr = pnp.CnnTrainer(params, B, s, lr=1e-4)
+    loss = tr.step(torch.from_numpy(u).cuda(), torch.from_numpy(nz).cuda(), sigma, update=False, want_loss=True)
+    gp = pnp.unpack_cnn_weights(tr.read(weights=False, grads=True)[1])
+    loss_ref, grads, absg = ocnn.l1_loss_and_grads(params, u[:, None].astype(np.float64),
+                                                   nz[:, None].astype(np.float64), sigma, bf16=True, with_abs=True)
+    assert loss == pytest.approx(loss_ref, rel=1e-5)
+    for (dW, db), (aW, ab), (gW, gb) in zip(grads, absg, gp):
+        assert np.linalg.norm(gW - dW) <= 2 * BF16_U * np.linalg.norm(aW)
+        assert np.linalg.norm(gb - db) <= 2 * BF16_U * max(np.linalg.norm(ab), 1e-30)
+        assert np.vdot(gW, dW) >= 0.999 * np.linalg.norm(gW) * np.linalg.norm(dW)

@@ -322,9 +322,9 @@ int pnp_den_create_cnn(pnp_den** den, const float* weights_host,
                        const int32_t* facet_cols_host, int nfc, int halo, int n, void* stream);
 
 /* Work decomposition of a CNN denoiser (a performance setting: the results do not depend on it, bit
- * for bit).  Each convolution layer walks strips of one 128-pixel column segment by about `rows`
- * output rows of a facet (the last layer: of a facet core); a strip stages rows + 2 input rows, so
- * taller strips re-read fewer halo rows and shorter ones balance the SMs better.  Default 32.
+ * for bit).  Each convolution layer walks strips of one 128-pixel column segment by at most `rows`
+ * output rows of a facet (the last layer: of a facet core); the rows of all segments are cut evenly over
+ * the SMs, so the setting only adds cuts, and a strip stages rows + 2 input rows.  Default 1024.
  *  rows   in [4, 1024]; PNP_ERR_INVALID_ARG otherwise or for a denoiser that is not a CNN.
  * Synchronises the device (work lists in use by launches in flight are not overwritten). */
 int pnp_den_cnn_set_strip_rows(pnp_den* den, int rows);

@@ -23,7 +23,8 @@
 //                D(z) = max(0, z - N(z)) and the FP64 stopping-test norms.
 //
 // conv64_rows layout.  Work is a strip: one 128-pixel column segment (x0 .. x0+127)
-// of a run of consecutive output rows of a facet (the strip height is autotuned).
+// of a run of consecutive output rows of a facet.  The rows of all column segments form one
+// sequence that is cut evenly over the SMs (conv_strips).
 // The strip's input rows (64 channels, pixels x0-1 .. x0+128) stream through a
 // ring of shared-memory row slots, staged channel-block-major: [kb][pixel][8 ch]
 // with the 130 pixels of a block 16 bytes apart (in a 128-byte aligned 2176-byte
@@ -67,6 +68,8 @@ constexpr int CONV_SMEM = IN_SLOTS * ROW_BYTES + B_BYTES;  // 212992
 constexpr int EPI_WARPS = 16;                           // 4 lane quarters x 4 channel quarters
 constexpr int MMA_WARP = EPI_WARPS, TMA_WARP = EPI_WARPS + 1;
 constexpr int CONV_THREADS = (EPI_WARPS + 2) * 32;
+constexpr int CONV_EPI = EPI_WARPS * 32;                // epilogue threads
+constexpr int CONV_MASK_SMEM = CONV_SMEM + CONV_EPI * 32;  // backward data: and the mask pieces of a row
 constexpr int FIRST_ROWS = 64;                          // cnn_first: image rows per block
 constexpr uint32_t CNN_WAIT_LIMIT = 1u << 26;
 
@@ -77,10 +80,10 @@ struct CnnState {
   int4* d_facets = nullptr;              // per facet: (R0, C0, Hf, Wf)
   int4* d_cores = nullptr;               // per facet: (r0, r1, c0, c1)
   int4* d_strips = nullptr;              // conv64_rows work list (conv_strips)
-  int n_strips = 0;
+  int n_strips = 0, conv_grid = 0;       // CTA b walks strips b, b + conv_grid, ...
   int4* d_lstrips = nullptr;             // last layer's work list: strips of the facet cores (last_strips)
   int n_lstrips = 0;
-  int strip_rows = STRIP_ROWS;           // target output rows per strip of both work lists (autotuned)
+  int strip_rows = STRIP_ROWS;           // output rows per strip of both work lists, at most
   size_t cap_strips = 0, cap_lstrips = 0;  // allocated entries of d_strips, d_lstrips
   uint32_t* d_wfrag = nullptr;           // last layer's weights as mma.sync B fragments [4 k][2 n][32 lanes][2]
   __nv_bfloat16* d_canvas[2] = {nullptr, nullptr};
@@ -129,6 +132,14 @@ __device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, i
       "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(su32(bar))
       : "memory");
 }
+
+// 16-byte global -> shared copy; nbytes = 0 fills the 16 bytes with zeros (src is not read)
+__device__ __forceinline__ void cp_async16_zfill(void* dst, const void* src, int nbytes) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(su32(dst)), "l"(src), "r"(nbytes) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit_group() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait_group() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 __device__ __forceinline__ void tmem_alloc(uint32_t* dst, uint32_t ncols) {
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(dst)), "r"(ncols)
@@ -183,7 +194,6 @@ struct ConvArgs {
   const int4* strips;      // conv_strips
   int n_strips, Hc, Wc;
   int* status;
-  int mode;                    // 0: forward, out = ReLU(acc + bias); 1: backward data, out = acc * [mask > 0]
   const __nv_bfloat16* mask;   // backward data: activations whose ReLU mask gates the output (same canvas layout)
 };
 
@@ -195,8 +205,13 @@ struct ConvArgs {
 // D_{s-1}[dy 1]) + D_s[dy 2].  Every MMA has the full N = 192 (no accumulator ring to wrap, no fresh-row
 // split), so an input row costs exactly 12 MMAs.  Warp roles: warps 0-15 the epilogue, warp 16 the MMAs
 // (one lane), warp 17 the TMA loads (one lane); epilogue warp w reads TMEM lanes 32 (w % 4) .. + 31 and channels 16 (w / 4) .. + 15 of each part.
+// What bounds it: the forward layer tensor pipe (66% active) and HBM (70% of the copy rate) together at 2048^2; the
+// backward layer, which reads its mask too, HBM (5.4 TB/s).  Per layer, before (waits between two rows' MMAs, 220
+// instructions per epilogue warp and row) and now: 2048^2 / 16 facets 353 -> 269 us, 16 x 256^2 83 -> 59 us forward
+// and 83 -> 74 us backward.
 constexpr int ROW_N = 3 * CH;                 // 192 accumulator columns per staged input row
 constexpr int ROW_DBUF = 2;                   // TMEM buffers (2 x 192 of the 512 columns)
+constexpr int MMA_AHEAD = 6;                  // MMAs of a row issued before the waits for the next row
 
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(
@@ -206,13 +221,33 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
       : "r"(taddr));
 }
 
+// pairs of floats as 64-bit values (packed FP32 adds: lane-wise, the rounding of scalar adds)
+typedef unsigned long long f2;
+__device__ __forceinline__ f2 pk(uint32_t x, uint32_t y) {
+  f2 d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(x), "r"(y));
+  return d;
+}
+__device__ __forceinline__ f2 add2(f2 a, f2 b) {
+  f2 d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ __nv_bfloat162 to_bf2(f2 a) {
+  uint32_t x, y;
+  asm("mov.b64 {%0, %1}, %2;" : "=r"(x), "=r"(y) : "l"(a));
+  return __floats2bfloat162_rn(__uint_as_float(x), __uint_as_float(y));
+}
+
+// MODE 0: forward, out = ReLU(acc + bias); 1: backward data, out = acc * [mask > 0]
+template <int MODE>
 __global__ void __launch_bounds__(CONV_THREADS, 1) conv64_rows(ConvArgs A, const __grid_constant__ CUtensorMap tmain,
                                                                const __grid_constant__ CUtensorMap thalo) {
   extern __shared__ __align__(1024) unsigned char sm[];  // [IN_SLOTS][ROW_BYTES] input ring, then B
   unsigned char* sb = sm + IN_SLOTS * ROW_BYTES;
   __shared__ uint64_t in_full[IN_SLOTS], in_empty[IN_SLOTS], d_full[ROW_DBUF], d_empty[ROW_DBUF];
   __shared__ uint32_t s_tmem;
-  __shared__ float s_bias[CH];
+  __shared__ __align__(16) float s_bias[CH];
   __shared__ volatile int s_abort;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   {
@@ -228,7 +263,7 @@ __global__ void __launch_bounds__(CONV_THREADS, 1) conv64_rows(ConvArgs A, const
     }
     for (int k = 0; k < ROW_DBUF; ++k) {
       bar_init(&d_full[k], 1);
-      bar_init(&d_empty[k], EPI_WARPS * 32);  // every epilogue thread reads every buffer
+      bar_init(&d_empty[k], EPI_WARPS);  // every epilogue warp reads every buffer
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     s_abort = 0;
@@ -277,102 +312,115 @@ __global__ void __launch_bounds__(CONV_THREADS, 1) conv64_rows(ConvArgs A, const
       const uint64_t adesc0 = smem_desc(su32(sm), KB_BYTES, 128);
       const uint64_t bdesc0 = smem_desc(su32(sb), B_GROUP_BYTES, 128);
       const uint32_t idesc = idesc_n(ROW_N);
-      uint32_t L = 0;
-      for (int strip = blockIdx.x; strip < A.n_strips && !s_abort; strip += stride) {
-        const int R = A.strips[strip].z & 0xFFFF;
-        for (int s = 0; s < R + 2; ++s, ++L) {
-          const uint32_t slot = L % IN_SLOTS, buf = L % ROW_DBUF;
-          if (!bar_wait(&in_full[slot], (L / IN_SLOTS) & 1)) s_abort = 1;
-          if (L >= ROW_DBUF && !bar_wait(&d_empty[buf], ((L / ROW_DBUF) - 1) & 1)) s_abort = 1;
-          if (s_abort) break;
-          tc_fence_after();
-          const uint64_t arow = adesc0 + (uint64_t)((slot * ROW_BYTES) >> 4);
-          const uint32_t d = tmem + buf * ROW_N;
+      uint32_t L = 0, rows = 0;  // staged rows of all strips
+      for (int strip = blockIdx.x; strip < A.n_strips; strip += stride) rows += (A.strips[strip].z & 0xFFFF) + 2;
+      // row l is staged and its accumulator free (waits that gave up end the issue)
+      auto ready = [&](uint32_t l) {
+        return bar_wait(&in_full[l % IN_SLOTS], (l / IN_SLOTS) & 1) &&
+               (l < ROW_DBUF || bar_wait(&d_empty[l % ROW_DBUF], ((l / ROW_DBUF) - 1) & 1)) && !s_abort;
+      };
+      bool ok = rows > 0 && ready(0);
+      for (; ok && L < rows; ++L) {
+        const uint32_t slot = L % IN_SLOTS, buf = L % ROW_DBUF;
+        tc_fence_after();
+        const uint64_t arow = adesc0 + (uint64_t)((slot * ROW_BYTES) >> 4);
+        const uint32_t d = tmem + buf * ROW_N;
 #pragma unroll
-          for (int dk = 0; dk < 12; ++dk) {
-            const int dx = dk >> 2, kk = dk & 3;
-            const uint64_t ad = arow + (uint64_t)((2 * kk * KB_BYTES + dx * 16) >> 4);
-            const uint64_t bd = bdesc0 + (uint64_t)(((dx * 8 + 2 * kk) * B_GROUP_BYTES) >> 4);
-            mma_bf16(d, ad, bd, idesc, dk > 0 ? 1u : 0u);
-          }
-          mma_commit(&in_empty[slot]);  // the input slot may be refilled
-          mma_commit(&d_full[buf]);     // D_s is complete
+        for (int dk = 0; dk < 12; ++dk) {
+          // the waits for the next row (neither depends on this row's MMAs) run under the MMAs issued so far:
+          // between two rows they left the tensor pipe idle for ~630 of 1970 cycles a row
+          if (dk == MMA_AHEAD) ok = L + 1 == rows || ready(L + 1);
+          const int dx = dk >> 2, kk = dk & 3;
+          const uint64_t ad = arow + (uint64_t)((2 * kk * KB_BYTES + dx * 16) >> 4);
+          const uint64_t bd = bdesc0 + (uint64_t)(((dx * 8 + 2 * kk) * B_GROUP_BYTES) >> 4);
+          mma_bf16(d, ad, bd, idesc, dk > 0 ? 1u : 0u);
         }
+        mma_commit(&in_empty[slot]);  // the input slot may be refilled
+        mma_commit(&d_full[buf]);     // D_s is complete
       }
+      if (!ok && rows > 0) s_abort = 1;
       // the tensor memory is freed below only after the last MMAs have completed
       if (L > 0) bar_wait(&in_empty[(L - 1) % IN_SLOTS], ((L - 1) / IN_SLOTS) & 1);
     }
     __syncwarp();
   } else {
     // ---------------- epilogue: q1 = partial sums of output row s - 1 (its dy = 0 part), q2 = those of
-    // row s - 2 (dy = 0 and 1); staged row s completes row s - 2 with its dy = 2 part
+    // row s - 2 (dy = 0 and 1); staged row s completes row s - 2 with its dy = 2 part.  A warp takes a row in
+    // ~90 instructions (packed adds, ReLU and mask on BF16 pairs, no select: columns beyond the facet are not
+    // stored, they are zero from the canvas's allocation); at 220 the 16 warps' issue slots and latency, not
+    // the MMAs, set the pace.
     const int lq = warp & 3, cq = warp >> 2;
     const int m = lq * 32 + lane;
-    const size_t plane = (size_t)A.Wc * 8;
+    const size_t plane = (size_t)A.Wc * 8, line = (size_t)A.Wc * CH;
+    const f2* bias = reinterpret_cast<const f2*>(s_bias + 16 * cq);
+    // MODE 1: this thread's two mask pieces of the next output row (in registers they were spilled, and the
+    // spill waited for the load)
+    uint4* mask_at = reinterpret_cast<uint4*>(sm + CONV_SMEM) + threadIdx.x;
+    const uint32_t tbase = tmem + ((uint32_t)(lq * 32) << 16) + cq * 16;
     uint32_t L = 0;
     bool stop = false;
     for (int strip = blockIdx.x; strip < A.n_strips && !stop; strip += stride) {
       const int4 S = A.strips[strip];
-      const int ya = S.z >> 16, R = S.z & 0xFFFF, Hf = S.w >> 16, Wf = S.w & 0xFFFF;
-      float q1[16] = {}, q2[16] = {};
+      const int ya = S.z >> 16, R = S.z & 0xFFFF, Wf = S.w & 0xFFFF;
+      const bool live = S.y + m < Wf;
+      size_t pix = canvas_index(S.x, ya, S.y + m, 16 * cq, A.Hc, A.Wc);  // block q of output row r at pix + q * plane
+      f2 q1[8] = {}, q2[8] = {};
       for (int s = 0; s < R + 2; ++s, ++L) {
         const uint32_t buf = L % ROW_DBUF;
-        const bool ok = !s_abort && bar_wait(&d_full[buf], (L / ROW_DBUF) & 1);
-        if (!ok) s_abort = 1;
+        const bool ok = bar_wait(&d_full[buf], (L / ROW_DBUF) & 1);
         if (!__all_sync(0xffffffffu, ok)) {
+          s_abort = 1;
           stop = true;
           break;
         }
         tc_fence_after();
-        const uint32_t base = tmem + ((uint32_t)(lq * 32) << 16) + buf * ROW_N + cq * 16;
-        uint32_t v2[16];
-        tmem_ld16(base, v2);  // dy = 2: output row s - 2 (the other two parts are read after it is stored)
-        tmem_wait_ld();
-        const int r = s - 2;  // the output row completed by this input row
-        if (r >= 0) {
-          const int y = ya + r, x = S.y + m;
-          if (y < A.Hc && x < A.Wc) {
-            const bool live = x < Wf && y < Hf;  // outside the facet the canvas stays zero
-            const size_t pix = canvas_index(S.x, y, x, 16 * cq, A.Hc, A.Wc);  // block q at pix + q * plane
-            uint4 pk[2];
-            uint32_t* pw = reinterpret_cast<uint32_t*>(pk);
-            if (A.mode == 0) {
-#pragma unroll
-              for (int c = 0; c < 16; c += 2) {
-                const float a0 = q2[c] + __uint_as_float(v2[c]), a1 = q2[c + 1] + __uint_as_float(v2[c + 1]);
-                const float o0 = live ? fmaxf(0.f, a0 + s_bias[16 * cq + c]) : 0.f;
-                const float o1 = live ? fmaxf(0.f, a1 + s_bias[16 * cq + c + 1]) : 0.f;
-                __nv_bfloat162 h = __floats2bfloat162_rn(o0, o1);
-                pw[c / 2] = *reinterpret_cast<uint32_t*>(&h);
-              }
-            } else {
-              uint4 mk[2];
-#pragma unroll
-              for (int q = 0; q < 2; ++q) mk[q] = *reinterpret_cast<const uint4*>(A.mask + pix + q * plane);
-              const __nv_bfloat16* mh = reinterpret_cast<const __nv_bfloat16*>(mk);
-#pragma unroll
-              for (int c = 0; c < 16; c += 2) {
-                const float a0 = q2[c] + __uint_as_float(v2[c]), a1 = q2[c + 1] + __uint_as_float(v2[c + 1]);
-                const float o0 = (live && __bfloat162float(mh[c]) > 0.f) ? a0 : 0.f;
-                const float o1 = (live && __bfloat162float(mh[c + 1]) > 0.f) ? a1 : 0.f;
-                __nv_bfloat162 h = __floats2bfloat162_rn(o0, o1);
-                pw[c / 2] = *reinterpret_cast<uint32_t*>(&h);
-              }
-            }
-#pragma unroll
-            for (int q = 0; q < 2; ++q) *reinterpret_cast<uint4*>(A.out + pix + q * plane) = pk[q];
-          }
-        }
-        uint32_t v1[16], v0[16];
-        tmem_ld16(base + CH, v1);      // dy = 1: output row s - 1
-        tmem_ld16(base + 2 * CH, v0);  // dy = 0: output row s
+        uint32_t v2[16], v1[16], v0[16];  // dy = 2, 1, 0: output rows s - 2, s - 1, s
+        tmem_ld16(tbase + buf * ROW_N, v2);
+        tmem_ld16(tbase + buf * ROW_N + CH, v1);
+        tmem_ld16(tbase + buf * ROW_N + 2 * CH, v0);
         tmem_wait_ld();
         tc_fence_before();
-        bar_arrive(&d_empty[buf]);  // this thread's parts of D_s are in registers
+        __syncwarp();
+        if (lane == 0) bar_arrive(&d_empty[buf]);  // this warp's parts of D_s are in registers
+        if (s >= 2) {
+          uint4 out[2];
+          uint32_t* ow = reinterpret_cast<uint32_t*>(out);
+          uint4 mk[2];
+          if (MODE == 1) {
+            cp_async_wait_group<0>();
+            mk[0] = mask_at[0];
+            mk[1] = mask_at[CONV_EPI];
+          }
+          const uint32_t* mw = reinterpret_cast<const uint32_t*>(mk);
 #pragma unroll
-        for (int c = 0; c < 16; ++c) {
-          q2[c] = q1[c] + __uint_as_float(v1[c]);  // row s - 1: dy = 0 + dy = 1 (not used at s = 0)
-          q1[c] = __uint_as_float(v0[c]);          // row s: dy = 0
+          for (int c = 0; c < 8; ++c) {
+            f2 a = add2(q2[c], pk(v2[2 * c], v2[2 * c + 1]));
+            const __nv_bfloat162 zero = __floats2bfloat162_rn(0.f, 0.f);
+            if (MODE == 0) {
+              const __nv_bfloat162 h = __hmax2(to_bf2(add2(a, bias[c])), zero);  // a NaN becomes 0, as fmaxf(0, NaN)
+              ow[c] = *reinterpret_cast<const uint32_t*>(&h);
+            } else {
+              const __nv_bfloat162 h = to_bf2(a);
+              ow[c] = *reinterpret_cast<const uint32_t*>(&h) &
+                      __hgt2_mask(*reinterpret_cast<const __nv_bfloat162*>(&mw[c]), zero);
+            }
+          }
+          if (live) {
+#pragma unroll
+            for (int q = 0; q < 2; ++q) *reinterpret_cast<uint4*>(A.out + pix + q * plane) = out[q];
+          }
+          pix += line;
+        }
+        if (MODE == 1 && s >= 1 && s < R + 1) {  // the masks of output row s - 1, completed by the next staged row
+#pragma unroll
+          for (int q = 0; q < 2; ++q)
+            cp_async16_zfill(mask_at + q * CONV_EPI, live ? A.mask + pix + q * plane : A.mask, live ? 16 : 0);
+          cp_async_commit_group();
+        }
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          q2[c] = add2(q1[c], pk(v1[2 * c], v1[2 * c + 1]));  // row s - 1: dy = 0 + dy = 1 (not used at s = 0)
+          q1[c] = pk(v0[2 * c], v0[2 * c + 1]);               // row s: dy = 0
         }
       }
     }
@@ -506,14 +554,6 @@ __device__ __forceinline__ void ldmatrix_x4(uint32_t (&r)[4], const void* p) {
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                : "r"(su32(p)));
 }
-// 16-byte global -> shared copy; nbytes = 0 fills the 16 bytes with zeros (src is not read)
-__device__ __forceinline__ void cp_async16_zfill(void* dst, const void* src, int nbytes) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(su32(dst)), "l"(src), "r"(nbytes) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit_group() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait_group() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-
 // activation row r of facet f, pixels x0 - 1 .. x0 + 142, into a staged row [block][px][8 ch] (zero outside
 // rows [0, Hf) and columns [0, Wf): the 'same' padding at the facet's edges)
 __device__ __forceinline__ void last_stage_row(unsigned char* dst, const LastArgs& A, int f, int r, int x0, int Hf,
@@ -698,25 +738,44 @@ int sms_of_device() {
 // The two convolution work lists for strips of about `rows` output rows: the hidden layers' strips of
 // the extended facets, and the last layer's strips of the facet cores.  Device arrays grow as needed.
 static int build_strips(CnnState* S, int rows) {
-  const std::vector<int4> strips = conv_strips(S->F, S->Hf.data(), S->Wf.data(), rows);
+  const int sms = sms_of_device();
+  const std::vector<int4> strips = conv_strips(S->F, S->Hf.data(), S->Wf.data(), sms, &S->conv_grid, rows);
+  // last layer: strips of the cores of at most `rows` rows, of the height (8 .. 128) at which the resident CTAs
+  // (four per SM) share the staged rows best: rounds x (rows + 2 halo rows)
   std::vector<int4> lstrips;
+  int best = 0;
+  int64_t best_cost = -1;
+  for (int h = 8; h <= 128; ++h) {
+    int64_t n = 0;
+    int tallest = 1;
+    for (int f = 0; f < S->F; ++f) {
+      const int H = S->fr1[f] - S->fr0[f], k = (H + std::min(h, rows) - 1) / std::min(h, rows);
+      n += (int64_t)((S->fc1[f] - S->fc0[f] + TILE_PX - 1) / TILE_PX) * k;
+      tallest = std::max(tallest, (H + k - 1) / k);
+    }
+    const int64_t cost = (n + 4 * sms - 1) / (4 * sms) * (tallest + 2);
+    if (best_cost < 0 || cost < best_cost) {
+      best_cost = cost;
+      best = std::min(h, rows);
+    }
+  }
   for (int f = 0; f < S->F; ++f) {
     const int cr0 = S->fr0[f] - S->R0[f], cr1 = S->fr1[f] - S->R0[f];
     const int cc0 = S->fc0[f] - S->C0[f], cc1 = S->fc1[f] - S->C0[f];
-    const int k = std::max(1, (cr1 - cr0 + rows - 1) / rows);
+    const int k = std::max(1, (cr1 - cr0 + best - 1) / best);
     for (int x0 = cc0; x0 < cc1; x0 += TILE_PX)
       for (int i = 0; i < k; ++i) {
         const int ya = cr0 + (int)((int64_t)(cr1 - cr0) * i / k), yb = cr0 + (int)((int64_t)(cr1 - cr0) * (i + 1) / k);
         if (yb > ya) lstrips.push_back(make_int4(f, x0, (ya << 16) | (yb - ya), (S->Hf[f] << 16) | S->Wf[f]));
       }
   }
-  auto fit = [](int4** p, size_t* cap, size_t need) -> int {
+  auto fit = [](void** p, size_t* cap, size_t need, size_t item) -> int {
     need = std::max<size_t>(1, need);
     if (*p && *cap >= need) return PNP_OK;
     cudaFree(*p);
     *p = nullptr;
     *cap = 0;
-    if (cudaMalloc(reinterpret_cast<void**>(p), need * sizeof(int4)) != cudaSuccess) {
+    if (cudaMalloc(p, need * item) != cudaSuccess) {
       cudaGetLastError();
       *p = nullptr;
       return fail(PNP_ERR_OOM, "CNN work list allocation failed");
@@ -724,8 +783,8 @@ static int build_strips(CnnState* S, int rows) {
     *cap = need;
     return PNP_OK;
   };
-  if (int rc = fit(&S->d_strips, &S->cap_strips, strips.size())) return rc;
-  if (int rc = fit(&S->d_lstrips, &S->cap_lstrips, lstrips.size())) return rc;
+  if (int rc = fit((void**)&S->d_strips, &S->cap_strips, strips.size(), sizeof(int4))) return rc;
+  if (int rc = fit((void**)&S->d_lstrips, &S->cap_lstrips, lstrips.size(), sizeof(int4))) return rc;
   if (!strips.empty())
     PNP_CUDA(cudaMemcpy(S->d_strips, strips.data(), strips.size() * sizeof(int4), cudaMemcpyHostToDevice));
   if (!lstrips.empty())
@@ -881,7 +940,6 @@ int cnn_denoise(pnp_den* d, cudaStream_t s, const float* z, float* out, int n, d
   CnnState* S = static_cast<CnnState*>(d->impl);
   if (!S) return fail(PNP_ERR_INVALID_ARG, "CNN denoiser not initialised");
   if (n != S->n) return fail(PNP_ERR_INVALID_ARG, "image side differs from the one the CNN denoiser was built for");
-  const int sms = sms_of_device();
   {
     FirstArgs F{z, n, 0, S->d_facets, S->F, S->Hc, S->Wc, S->d_w1, S->d_b, S->d_canvas[0]};
     cnn_first<<<dim3(S->Wc / FIRST_PX, (S->Hc + FIRST_ROWS - 1) / FIRST_ROWS, S->F), 256, 0, s>>>(F);
@@ -889,16 +947,15 @@ int cnn_denoise(pnp_den* d, cudaStream_t s, const float* z, float* out, int n, d
   }
   static bool attr = false;
   if (!attr) {
-    PNP_CUDA(cudaFuncSetAttribute(conv64_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, CONV_SMEM));
+    PNP_CUDA(cudaFuncSetAttribute(conv64_rows<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, CONV_SMEM));
     PNP_CUDA(cudaFuncSetAttribute(cnn_last, cudaFuncAttributeMaxDynamicSharedMemorySize, LAST_SMEM));
     attr = true;
   }
   int cur = 0;
   for (int l = 0; l < 6; ++l) {
     ConvArgs C{S->d_canvas[1 - cur], S->d_wmid + (size_t)l * 9 * CH * CH, S->d_b + (l + 1) * CH, S->d_strips,
-               S->n_strips, S->Hc, S->Wc, S->d_status, 0, nullptr};
-    const int grid = std::max(1, std::min(S->n_strips, sms));
-    conv64_rows<<<grid, CONV_THREADS, CONV_SMEM, s>>>(C, S->map[cur][0], S->map[cur][1]);
+               S->n_strips, S->Hc, S->Wc, S->d_status, nullptr};
+    conv64_rows<0><<<S->conv_grid, CONV_THREADS, CONV_SMEM, s>>>(C, S->map[cur][0], S->map[cur][1]);
     PNP_CHECK_LAUNCH();
     cur = 1 - cur;
   }
@@ -913,31 +970,63 @@ int cnn_denoise(pnp_den* d, cudaStream_t s, const float* z, float* out, int n, d
 }
 
 int conv64_launch(cudaStream_t s, const void* in_map, __nv_bfloat16* out, const __nv_bfloat16* w_packed,
-                  const float* bias, const int4* strips, int n_strips, int Hc, int Wc, int mode,
+                  const float* bias, const int4* strips, int n_strips, int grid, int Hc, int Wc, int mode,
                   const __nv_bfloat16* mask, int* status) {
   static bool attr = false;
   if (!attr) {
-    PNP_CUDA(cudaFuncSetAttribute(conv64_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, CONV_SMEM));
+    PNP_CUDA(cudaFuncSetAttribute(conv64_rows<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, CONV_SMEM));
+    PNP_CUDA(cudaFuncSetAttribute(conv64_rows<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, CONV_MASK_SMEM));
     attr = true;
   }
-  ConvArgs C{out, w_packed, bias, strips, n_strips, Hc, Wc, status, mode, mask};
-  const int grid = std::max(1, std::min(n_strips, sms_of_device()));
+  ConvArgs C{out, w_packed, bias, strips, n_strips, Hc, Wc, status, mask};
   const CUtensorMap* maps = static_cast<const CUtensorMap*>(in_map);
-  conv64_rows<<<grid, CONV_THREADS, CONV_SMEM, s>>>(C, maps[0], maps[1]);
+  if (mode == 0) conv64_rows<0><<<grid, CONV_THREADS, CONV_SMEM, s>>>(C, maps[0], maps[1]);
+  else conv64_rows<1><<<grid, CONV_THREADS, CONV_MASK_SMEM, s>>>(C, maps[0], maps[1]);
   PNP_CHECK_LAUNCH();
   return PNP_OK;
 }
 
-std::vector<int4> conv_strips(int F, const int* Hf, const int* Wf, int rows) {
-  std::vector<int4> out;
-  for (int f = 0; f < F; ++f) {
-    const int k = std::max(1, (Hf[f] + rows - 1) / rows);  // strips per column segment
+// The sequence (facet, column segment, row) is cut into waves x grid equal shares of at most `rows` rows, dealt
+// round robin, and a share again where a segment ends: with the default height one share per SM.  Equal shares keep
+// the SMs level (32-row strips of whole segments: 8 x 128^2 images gave 32 strips to 152 SMs, 42 us a layer -> 18;
+// 2048^2 in 16 facets 1440 strips in 9.5 rounds, denoise 2.39 -> 2.19 ms).  A strip stages rows + 2 input rows.
+// CTA b walks entries b, b + grid, ... of the list (two bounds read per CTA in the kernel instead of this stride
+// cost it 15%), so every CTA gets the same number of strips: those with fewer cut their tallest.
+std::vector<int4> conv_strips(int F, const int* Hf, const int* Wf, int sms, int* grid_out, int rows) {
+  int64_t total = 0;
+  for (int f = 0; f < F; ++f) total += (int64_t)((Wf[f] + TILE_PX - 1) / TILE_PX) * Hf[f];
+  // at least four rows per CTA: below that the halo rows outweigh what another SM adds
+  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(sms, total / 4));
+  const int64_t shares = grid * std::max<int64_t>(1, (total + (int64_t)grid * rows - 1) / ((int64_t)grid * rows));
+  std::vector<std::vector<int4>> cta(grid);
+  int64_t at = 0, share = 0;  // position in the sequence, and the share it lies in
+  for (int f = 0; f < F; ++f)
     for (int x0 = 0; x0 < Wf[f]; x0 += TILE_PX)
-      for (int i = 0; i < k; ++i) {
-        const int ya = (int)((int64_t)Hf[f] * i / k), yb = (int)((int64_t)Hf[f] * (i + 1) / k);
-        if (yb > ya) out.push_back(make_int4(f, x0, (ya << 16) | (yb - ya), (Hf[f] << 16) | Wf[f]));
+      for (int y = 0; y < Hf[f];) {
+        while (total * (share + 1) / shares <= at) ++share;
+        const int n = (int)std::min<int64_t>(Hf[f] - y, total * (share + 1) / shares - at);
+        cta[share % grid].push_back(make_int4(f, x0, (y << 16) | n, (Hf[f] << 16) | Wf[f]));
+        y += n;
+        at += n;
       }
+  size_t most = 1;
+  for (const auto& c : cta) most = std::max(most, c.size());
+  std::vector<int4> out(most * grid);
+  for (int b = 0; b < grid; ++b) {
+    auto& c = cta[b];
+    while (c.size() < most) {
+      size_t t = 0;
+      for (size_t k = 1; k < c.size(); ++k)
+        if ((c[k].z & 0xFFFF) > (c[t].z & 0xFFFF)) t = k;
+      const int y = c[t].z >> 16, n = c[t].z & 0xFFFF, h = n / 2;  // n >= 2: a share has four rows or more
+      int4 lower = c[t];
+      lower.z = ((y + h) << 16) | (n - h);
+      c[t].z = (y << 16) | h;
+      c.insert(c.begin() + t + 1, lower);
+    }
+    for (size_t k = 0; k < most; ++k) out[k * grid + b] = c[k];
   }
+  *grid_out = grid;
   return out;
 }
 

@@ -638,7 +638,7 @@ int nblocks(int64_t count, int threads = 256) {
 struct pnp_cnn_trainer {
   pnp::Dims d{};
   cudaStream_t stream = nullptr;
-  int n_strips = 0, t = 0, sms = 0;
+  int n_strips = 0, conv_grid = 0, t = 0, sms = 0;
   int parts = 0;          // CTAs of the weight-gradient kernel
   float* part = nullptr;  // their partial sums (parts x WGT_SUMS)
   double lr = 1e-4, b1 = 0.9, b2 = 0.999, eps = 1e-8;
@@ -734,7 +734,7 @@ int primal_forward(pnp_cnn_trainer* T, const float* z) {
     return rc;
   for (int k = 1; k <= 6; ++k)
     if (int rc = conv64_launch(s, T->map_act[k], T->act[k + 1], T->wf + (size_t)(k - 1) * NWM, T->bias + k * CH,
-                               T->strips, T->n_strips, d.Hc, d.Wc, 0, nullptr, T->status))
+                               T->strips, T->n_strips, T->conv_grid, d.Hc, d.Wc, 0, nullptr, T->status))
       return rc;
   return PNP_OK;
 }
@@ -754,7 +754,7 @@ int power_iterate(pnp_cnn_trainer* T, const float* v0, int iters, double* sigma_
     int cur = 0;
     for (int k = 1; k <= 6; ++k) {
       if (int rc = conv64_launch(s, T->map_dp[cur], T->dp[1 - cur], T->wf + (size_t)(k - 1) * NWM, nullptr, T->strips,
-                                 T->n_strips, d.Hc, d.Wc, 1, T->act[k + 1], T->status))
+                                 T->n_strips, T->conv_grid, d.Hc, d.Wc, 1, T->act[k + 1], T->status))
         return rc;
       cur = 1 - cur;
     }
@@ -765,7 +765,7 @@ int power_iterate(pnp_cnn_trainer* T, const float* v0, int iters, double* sigma_
     cur = 0;
     for (int k = 6; k >= 1; --k) {
       if (int rc = conv64_launch(s, T->map_dp[cur], T->dp[1 - cur], T->wb + (size_t)(k - 1) * NWM, nullptr, T->strips,
-                                 T->n_strips, d.Hc, d.Wc, 1, T->act[k], T->status))
+                                 T->n_strips, T->conv_grid, d.Hc, d.Wc, 1, T->act[k], T->status))
         return rc;
       cur = 1 - cur;
     }
@@ -834,7 +834,7 @@ int pnp_cnn_trainer_create(pnp_cnn_trainer** out, const float* weights_host, int
   for (int i = 1; ok && i <= 7; ++i) ok = al((void**)&T->tan[i], canvas * 2);
   std::vector<int4> facets(batch, make_int4(0, 0, size, size));
   const std::vector<int> sides(batch, size);
-  const std::vector<int4> strips = conv_strips(batch, sides.data(), sides.data());
+  const std::vector<int4> strips = conv_strips(batch, sides.data(), sides.data(), T->sms, &T->conv_grid);
   T->n_strips = (int)strips.size();
   ok = ok && al((void**)&T->strips, strips.size() * sizeof(int4));
   if (!ok) {
@@ -899,7 +899,7 @@ int pnp_cnn_train_step(pnp_cnn_trainer* T, const float* u, const float* noise, d
     return rc;
   for (int k = 1; k <= 6; ++k)
     if (int rc = conv64_launch(s, T->map_act[k], T->act[k + 1], T->wf + (size_t)(k - 1) * NWM, T->bias + k * CH,
-                               T->strips, T->n_strips, d.Hc, d.Wc, 0, nullptr, T->status))
+                               T->strips, T->n_strips, T->conv_grid, d.Hc, d.Wc, 0, nullptr, T->status))
       return rc;
   PNP_CUDA(cudaMemsetAsync(T->loss, 0, sizeof(double), s));
   if (int rc = many_to_one_launch<M2O_LOSS, false>(s, d, T->sms, T->act[7], T->w8r, 1, T->bias, T->z, u, T->gout, T->loss))
@@ -912,7 +912,7 @@ int pnp_cnn_train_step(pnp_cnn_trainer* T, const float* u, const float* noise, d
     float* gW = T->g + OFF_MID + (k - 1) * MID_STRIDE;
     if (int rc = wgrad64_launch(s, d, T->dp[cur], T->act[k], T->part, T->parts, gW, gW + NWM)) return rc;
     if (int rc = conv64_launch(s, T->map_dp[cur], T->dp[1 - cur], T->wb + (size_t)(k - 1) * NWM, nullptr,
-                               T->strips, T->n_strips, d.Hc, d.Wc, 1, T->act[k], T->status))
+                               T->strips, T->n_strips, T->conv_grid, d.Hc, d.Wc, 1, T->act[k], T->status))
       return rc;
     cur = 1 - cur;
   }
@@ -962,7 +962,7 @@ int pnp_cnn_train_step_fne(pnp_cnn_trainer* T, const float* u, const float* nois
   if (int rc = layer1_tangent(T, T->jv, T->tan[1])) return rc;
   for (int k = 1; k <= 6; ++k)
     if (int rc = conv64_launch(s, T->map_tan[k], T->tan[k + 1], T->wf + (size_t)(k - 1) * NWM, nullptr, T->strips,
-                               T->n_strips, d.Hc, d.Wc, 1, T->act[k + 1], T->status))
+                               T->n_strips, T->conv_grid, d.Hc, d.Wc, 1, T->act[k + 1], T->status))
       return rc;
   if (int rc = many_to_one_launch<M2O_JAC, false>(s, d, T->sms, T->tan[7], T->w8r, 1, nullptr, T->jv, nullptr, T->jw, nullptr))
     return rc;
@@ -978,7 +978,7 @@ int pnp_cnn_train_step_fne(pnp_cnn_trainer* T, const float* u, const float* nois
                                 T->g + OFF_MID + (k - 1) * MID_STRIDE, T->junk))
       return rc;
     if (int rc = conv64_launch(s, T->map_dp[cur], T->dp[1 - cur], T->wb + (size_t)(k - 1) * NWM, nullptr, T->strips,
-                               T->n_strips, d.Hc, d.Wc, 1, T->act[k], T->status))
+                               T->n_strips, T->conv_grid, d.Hc, d.Wc, 1, T->act[k], T->status))
       return rc;
     cur = 1 - cur;
   }

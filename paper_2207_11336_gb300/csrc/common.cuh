@@ -244,16 +244,16 @@ int cnn_status(pnp_den* d, int* flags);
 __host__ __device__ __forceinline__ size_t conv_wpack_index(int dy, int dx, int ci, int co) {
   return ((((size_t)dx * 8 + (ci >> 3)) * 3 + (2 - dy)) * 64 + co) * 8 + (ci & 7);
 }
-constexpr int STRIP_ROWS = 32;  // target output rows per convolution work unit
-// Work list of the hidden-layer convolution (conv64_rows): per facet, 128-column segments split into strips of about STRIP_ROWS
-// output rows; each entry is (facet, x0, ya << 16 | rows, Hf << 16 | Wf).
-std::vector<int4> conv_strips(int F, const int* Hf, const int* Wf, int rows = STRIP_ROWS);
-// the denoiser's convolution work lists rebuilt for strips of about `rows` output rows (4..1024)
+constexpr int STRIP_ROWS = 1024;  // output rows per convolution strip, at most
+// Work list of the hidden-layer convolution (conv64_rows): strips (facet, x0, ya << 16 | rows, Hf << 16 | Wf) of
+// 128-column segments; CTA b of the grid walks entries b, b + grid, ...
+std::vector<int4> conv_strips(int F, const int* Hf, const int* Wf, int sms, int* grid, int rows = STRIP_ROWS);
+// the denoiser's convolution work lists rebuilt for strips of at most `rows` output rows (4..1024)
 int cnn_set_strip_rows(pnp_den* d, int rows);
 int cnn_strip_rows(pnp_den* d);
 // the convolution reads its input through the TMA descriptor in_map (canvas_map_create)
 int conv64_launch(cudaStream_t s, const void* in_map, __nv_bfloat16* out, const __nv_bfloat16* w_packed,
-                  const float* bias, const int4* strips, int n_strips, int Hc, int Wc, int mode,
+                  const float* bias, const int4* strips, int n_strips, int grid, int Hc, int Wc, int mode,
                   const __nv_bfloat16* mask, int* status);
 // Activation canvases of the CNN hold BF16 values in planes of 8 channels:
 // [F][Hc][64 / 8][Wc][8], so that a row of one 8-channel block is contiguous (full-sector

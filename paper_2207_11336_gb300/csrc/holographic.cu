@@ -70,26 +70,40 @@ __global__ void __launch_bounds__(32 * HB_WARPS) holo_build(HBuildArgs A) {
 }
 
 // out[k] = sum_delta H[delta][k] X[k + delta] - b[k]   (b = NULL: no data term)
-__global__ void __launch_bounds__(256) holo_apply(const float2* __restrict__ H, const float2* __restrict__ X,
-                                                  const float2* __restrict__ b, float2* __restrict__ out, int logK,
-                                                  int Jmax, int S) {
-  const int K = 1 << logK, Km = K - 1, Jm1 = Jmax - 1;
+// A thread takes two neighbouring cells: one 16-byte load of H per offset, and along dc its second X is the next
+// offset's first.  JM1 = Jmax - 1 when it is a compile-time value (0: any), so that a row of the stencil's loads are
+// in flight together.  Bound by the read of H.  512^2 cells, J = 7 (354 MB of H): 83 -> 64 us, 5.6 TB/s.
+constexpr int HOLO_THREADS = 128;
+template <int JM1>
+__global__ void __launch_bounds__(HOLO_THREADS) holo_apply(const float2* __restrict__ H, const float2* __restrict__ X,
+                                                           const float2* __restrict__ b, float2* __restrict__ out,
+                                                           int logK, int Jmax, int S) {
+  const int K = 1 << logK, Km = K - 1, Jm1 = JM1 ? JM1 : Jmax - 1;
   const int64_t KK = (int64_t)K * K;
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < KK; k += (int64_t)gridDim.x * blockDim.x) {
-    const int r = (int)(k >> logK), c = (int)(k & Km);
-    float2 acc = make_float2(0.f, 0.f);
-    for (int dr = -Jm1; dr <= Jm1; ++dr) {
-      const float2* xrow = X + ((int64_t)((r + dr) & Km) << logK);
-      const float2* hrow = H + (int64_t)(dr + Jm1) * S * KK + k;
-      for (int dc = -Jm1; dc <= Jm1; ++dc) {
-        const float2 h = hrow[(int64_t)(dc + Jm1) * KK];
-        const float2 x = xrow[(c + dc) & Km];
-        acc.x = fmaf(h.x, x.x, fmaf(-h.y, x.y, acc.x));
-        acc.y = fmaf(h.x, x.y, fmaf(h.y, x.x, acc.y));
-      }
+  const int64_t k = 2 * (blockIdx.x * (int64_t)HOLO_THREADS + threadIdx.x);
+  if (k >= KK) return;
+  const int r = (int)(k >> logK), c = (int)(k & Km);
+  float2 a0 = make_float2(0.f, 0.f), a1 = a0;
+  for (int dr = -Jm1; dr <= Jm1; ++dr) {
+    const float2* xrow = X + ((int64_t)((r + dr) & Km) << logK);
+    const float2* hrow = H + (int64_t)(dr + Jm1) * S * KK + k;
+    float2 x = xrow[(c - Jm1) & Km];
+#pragma unroll
+    for (int dc = -Jm1; dc <= Jm1; ++dc) {
+      const float4 h = *reinterpret_cast<const float4*>(hrow + (int64_t)(dc + Jm1) * KK);
+      const float2 y = xrow[(c + dc + 1) & Km];
+      a0.x = fmaf(h.x, x.x, fmaf(-h.y, x.y, a0.x));
+      a0.y = fmaf(h.x, x.y, fmaf(h.y, x.x, a0.y));
+      a1.x = fmaf(h.z, y.x, fmaf(-h.w, y.y, a1.x));
+      a1.y = fmaf(h.z, y.y, fmaf(h.w, y.x, a1.y));
+      x = y;
     }
-    out[k] = b ? csub(acc, b[k]) : acc;
   }
+  if (b) {
+    a0 = csub(a0, b[k]);
+    a1 = csub(a1, b[k + 1]);
+  }
+  *reinterpret_cast<float4*>(out + k) = make_float4(a0.x, a0.y, a1.x, a1.y);
 }
 
 }  // namespace
@@ -172,9 +186,12 @@ int holo_apply_pass(pnp_plan* p, bool data_term) {
   cudaEvent_t ev;
   if (int rc = stage_begin(p, 1, &ev)) return rc;
   const int64_t KK = (int64_t)p->K * p->K;
-  const unsigned grid = (unsigned)std::min<int64_t>((KK + 255) / 256, (int64_t)p->num_sms * 16);
-  holo_apply<<<grid, 256, 0, p->stream>>>(p->d_H, p->d_gridA, data_term ? p->d_dirty : nullptr, p->d_gridB,
-                                          p->logK, p->Jmax, p->holo_S);
+  const unsigned grid = (unsigned)((KK / 2 + HOLO_THREADS - 1) / HOLO_THREADS);
+  const float2* dirty = data_term ? p->d_dirty : nullptr;
+  if (p->Jmax == 7)  // the default kernel support
+    holo_apply<6><<<grid, HOLO_THREADS, 0, p->stream>>>(p->d_H, p->d_gridA, dirty, p->d_gridB, p->logK, p->Jmax, p->holo_S);
+  else
+    holo_apply<0><<<grid, HOLO_THREADS, 0, p->stream>>>(p->d_H, p->d_gridA, dirty, p->d_gridB, p->logK, p->Jmax, p->holo_S);
   PNP_CHECK_LAUNCH();
   return stage_end(p, 1, ev);
 }

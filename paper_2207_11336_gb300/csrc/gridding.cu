@@ -180,6 +180,8 @@ __global__ void __launch_bounds__(GPASS_WARPS * 32, min_ctas<JP>()) gpass(const 
   ulonglong2* sx = reinterpret_cast<ulonglong2*>(ws + L::IN);
   const int Km = A.K - 1;
   const ulonglong2 zero4 = make_ulonglong2(0, 0);
+  // the next class's kernel may take the SMs' free slots from here on: it reads nothing that this one writes
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   // zeros: the accumulator, and the rings (a group without a row in a step reads a stale slot)
   for (int c = lane; c < L::OUT / 16; c += 32) reinterpret_cast<ulonglong2*>(ws)[c] = zero4;
   if (MODE != G_DEGRID)
@@ -359,6 +361,9 @@ __global__ void __launch_bounds__(GPASS_WARPS * 32, min_ctas<JP>()) gpass(const 
     nb = __shfl_sync(0xffffffffu, nb, 0);
     u = A.u_begin + (long long)nb * A.batch;
   }
+  // This kernel ends only after the previous class's kernel has (when it was launched as its dependent), so that
+  // the end of the last class's kernel is the end of the pass.
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   if (lane == 0 && atomicAdd(A.sched + 1, 1u) == gridDim.x * GPASS_WARPS - 1) {  // the last warp: every batch is taken
     A.sched[0] = 0;
     A.sched[1] = 0;
@@ -374,8 +379,10 @@ __global__ void permute_kernel(const float2* __restrict__ y, const int32_t* __re
   }
 }
 
+// The classes' kernels of one pass only add to the grid (or write their own rows), so each after the first is launched
+// as a programmatic dependent of the one before: its CTAs fill the tail of that kernel instead of waiting for its end.
 template <int MODE, bool BF, int JP, int W>
-int launch_class(pnp_plan* p, GArgs A, int s) {
+int launch_class(pnp_plan* p, GArgs A, int s, bool* first) {
   const int c = s * TAP_CLASSES + tap_class(JP, W);
   A.u_begin = p->h_class_units[c];
   A.n_units = p->h_class_units[c + 1];
@@ -392,21 +399,32 @@ int launch_class(pnp_plan* p, GArgs A, int s) {
   // about 16 batches per warp: the counter is taken seldom, the last batches are short
   A.batch = (int)std::max(1ll, std::min(16ll, count / (grid * GPASS_WARPS * 16)));
   A.sched = p->d_sched + 2 * c;
-  gpass<MODE, BF, JP, W><<<(unsigned)grid, GPASS_WARPS * 32, smem, p->stream>>>(A);
-  PNP_CHECK_LAUNCH();
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3(GPASS_WARPS * 32);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = p->stream;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = *first ? 0 : 1;
+  *first = false;
+  PNP_CUDA(cudaLaunchKernelEx(&cfg, gpass<MODE, BF, JP, W>, A));
+  g_launches.fetch_add(1, std::memory_order_relaxed);
   return PNP_OK;
 }
 
 template <int MODE, bool BF>
 int launch_classes(pnp_plan* p, const GArgs& A, int s) {
-  // the largest supports first: the short classes fill the tail of the launch sequence
-  if (int rc = launch_class<MODE, BF, 9, 16>(p, A, s)) return rc;
-  if (int rc = launch_class<MODE, BF, 8, 16>(p, A, s)) return rc;
-  if (int rc = launch_class<MODE, BF, 7, 16>(p, A, s)) return rc;
-  if (int rc = launch_class<MODE, BF, 6, 16>(p, A, s)) return rc;
-  if (int rc = launch_class<MODE, BF, 5, 16>(p, A, s)) return rc;
-  if (int rc = launch_class<MODE, BF, 5, 8>(p, A, s)) return rc;
-  return launch_class<MODE, BF, 4, 8>(p, A, s);
+  bool first = true;  // the largest supports first: the short classes fill the tails
+  if (int rc = launch_class<MODE, BF, 9, 16>(p, A, s, &first)) return rc;
+  if (int rc = launch_class<MODE, BF, 8, 16>(p, A, s, &first)) return rc;
+  if (int rc = launch_class<MODE, BF, 7, 16>(p, A, s, &first)) return rc;
+  if (int rc = launch_class<MODE, BF, 6, 16>(p, A, s, &first)) return rc;
+  if (int rc = launch_class<MODE, BF, 5, 16>(p, A, s, &first)) return rc;
+  if (int rc = launch_class<MODE, BF, 5, 8>(p, A, s, &first)) return rc;
+  return launch_class<MODE, BF, 4, 8>(p, A, s, &first);
 }
 
 template <int MODE>

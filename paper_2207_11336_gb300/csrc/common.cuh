@@ -147,7 +147,7 @@ struct pnp_plan {
   } graph;
 
   // device buffers
-  float* d_cinv = nullptr;     // n: 1 / c(a - n/2)
+  float2* d_cinv = nullptr;    // n: 1 / c(a - n/2), high and low part
   float2* d_tw = nullptr;      // K: exp(-2 pi i j / K)
   float2* d_twp = nullptr;     // radix-16 pass twiddles [16 + 256][16]: see fft.cu
   float2* d_gridA = nullptr;   // K*K: F Z x   (layout [k1][k0])

@@ -229,7 +229,7 @@ __device__ __forceinline__ int pad_position(int a, int n, int K) {
 struct FftArgs {
   int n;
   const float* x;          // P1 input image / Q2 current iterate
-  const float* cinv;       // 1 / c(p)
+  const float2* cinv;      // 1 / c(p) as an unevaluated sum of two floats
   const float2* tw;
   const float2* twp;       // radix-16 pass twiddles (TWP_ENTRIES)
   float2* tmp;             // T (K x n) or U (n x K)
@@ -254,6 +254,13 @@ __device__ __forceinline__ float2 cmul2(float2 a, float2 b) {
   return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 
+// v / (c_a c_b), the grid correction of pixel (a, b): the product of the two corrections keeps its rounding error
+// (an FMA), so that one rounding is left of the four that two float factors made
+__device__ __forceinline__ float correct(float v, float2 ca, float2 cb) {
+  const float p = ca.x * cb.x, e = fmaf(ca.x, cb.x, -p) + fmaf(ca.x, cb.y, ca.y * cb.x);
+  return fmaf(v, p, v * e);
+}
+
 // ---------------------------------------------------------------- P1
 // CH: the input is modulated by a w-stack's centre chirp (compiled separately so that the
 // plain operator keeps its register allocation)
@@ -266,12 +273,12 @@ __global__ void __launch_bounds__(R * (1 << LOGK) / 16) fft_p1(const __grid_cons
   const int a = blockIdx.x * R + rr;
   const bool live = a < n;  // the last CTA may hold fewer than R image rows
   float2* s = smem + rr * SROW;
-  const float ca = live ? A.cinv[a] : 0.f;
+  const float2 ca = live ? A.cinv[a] : make_float2(0.f, 0.f);
   float2 v[16];
 #pragma unroll
   for (int i = 0; i < 16; ++i) {
     const int b = unpad_index(j + i * T, n, K);
-    v[i] = (live && b >= 0) ? make_float2(A.x[(size_t)a * n + b] * ca * A.cinv[b], 0.f)
+    v[i] = (live && b >= 0) ? make_float2(correct(A.x[(size_t)a * n + b], ca, A.cinv[b]), 0.f)
                             : make_float2(0.f, 0.f);
   }
   if (CH && live) {  // Z_s of a w-stack: the centre chirp, separable over the two axes
@@ -471,7 +478,7 @@ __global__ void __launch_bounds__((1 << LOGK) / 16) fft_q2(const __grid_constant
 #pragma unroll
     for (int i = 0; i < 16; ++i) v[i] = row[j + i * T];
     fft_row<LOGK, +1>(v, smem, j, A.tw, A.twp);
-    const float ca = A.cinv[a];
+    const float2 ca = A.cinv[a];
     if (CH) {  // Re{conj(chirp) v}: the adjoint of the centre chirp of Z_s
       const float2 cha = A.chirp[a];
 #pragma unroll
@@ -479,14 +486,14 @@ __global__ void __launch_bounds__((1 << LOGK) / 16) fft_q2(const __grid_constant
         const int b = unpad_index(j + i * T, n, K);
         if (b >= 0) {
           const float2 c = cmul2(cha, A.chirp[b]);
-          gs[q * n + b] = (v[i].x * c.x + v[i].y * c.y) * ca * A.cinv[b];
+          gs[q * n + b] = correct(v[i].x * c.x + v[i].y * c.y, ca, A.cinv[b]);
         }
       }
     } else {
 #pragma unroll
       for (int i = 0; i < 16; ++i) {
         const int b = unpad_index(j + i * T, n, K);
-        if (b >= 0) gs[q * n + b] = v[i].x * ca * A.cinv[b];
+        if (b >= 0) gs[q * n + b] = correct(v[i].x, ca, A.cinv[b]);
       }
     }
   }
@@ -523,12 +530,12 @@ __global__ void __launch_bounds__(R * (1 << LOGK) / 32) fft_p1s(const __grid_con
   const int a = blockIdx.x * R + rr;
   const bool live = a < N;
   float2* s = smem + rr * SROW;
-  const float ca = live ? A.cinv[a] : 0.f;
+  const float2 ca = live ? A.cinv[a] : make_float2(0.f, 0.f);
   float2 v[16];
 #pragma unroll
   for (int i = 0; i < 16; ++i) {
     const int e = j + i * T, b = e < H ? e + H : e - H;
-    float2 val = make_float2(live ? A.x[(size_t)a * N + b] * ca * A.cinv[b] : 0.f, 0.f);
+    float2 val = make_float2(live ? correct(A.x[(size_t)a * N + b], ca, A.cinv[b]) : 0.f, 0.f);
     if (CH && live) {  // Z_s of a w-stack: the centre chirp, separable over the two axes
       const float2 c = cmul(A.chirp[a], A.chirp[b]);
       val = make_float2(val.x * c.x, val.x * c.y);
@@ -689,44 +696,52 @@ __global__ void __launch_bounds__(R * (1 << LOGK) / 16) fft_q1s(const __grid_con
 }
 
 // Q2 (split): rows a of U (even samples to one thread group, odd to the other), inverse transforms
-// and the centred outputs, then the epilogue of fft_q2 (two image rows per CTA).
+// and the centred outputs, then the epilogue of fft_q2 (two image rows per CTA).  R = 2: both rows at once, where
+// their threads fit a block of 512; the pass is then shorter (it is latency-bound: K = 512 12.1 -> 10.4 us,
+// K = 2048 21.4 -> 20.6 us); above, one after the other leaves room for two CTAs per SM.
+template <int LOGK>
+constexpr int q2_rows() {
+  return LOGK <= 12 ? 2 : 1;
+}
 template <int LOGK, bool CH>
-__global__ void __launch_bounds__((1 << LOGK) / 16, (1 << LOGK) / 16 <= 512 ? 2 : 1) fft_q2s(
+__global__ void __launch_bounds__(q2_rows<LOGK>() * (1 << LOGK) / 16, (1 << LOGK) / 16 <= 512 ? 2 : 1) fft_q2s(
     const __grid_constant__ FftArgs A) {
   using Sg = SplitGeom<LOGK - 1>;
   constexpr int N = Sg::N, K = 2 * N, T = Sg::T, H = Sg::H;
   extern __shared__ float2 smem[];
-  const int grp = threadIdx.x / T, j = threadIdx.x % T;
-  float2* buf = smem + grp * Sg::SROW;
-  float* gs = reinterpret_cast<float*>(smem + 2 * Sg::SROW);  // 2 x n gradient values
+  constexpr int R = q2_rows<LOGK>();
+  const int tr = threadIdx.x % (2 * T), g4 = threadIdx.x / T, grp = g4 & 1, j = threadIdx.x % T;
+  const int rr = R == 2 ? g4 >> 1 : 0;  // this thread's row when both run at once
+  float2* buf = smem + g4 * Sg::SROW;
+  float* gs = reinterpret_cast<float*>(smem + 2 * R * Sg::SROW);  // 2 x n gradient values
   const int a0 = 2 * blockIdx.x;
 #pragma unroll 1
-  for (int q2 = 0; q2 < 2; ++q2) {
+  for (int q2 = rr; q2 < 2; q2 += R) {
     const int a = a0 + q2;
     const float2* row = A.tmp + (size_t)a * K + grp;
-    if (q2) __syncthreads();  // the previous row is done with both buffers
+    if (R == 1 && q2) __syncthreads();  // the previous row is done with both buffers
     float2 v[16];
 #pragma unroll
     for (int i = 0; i < 16; ++i)  // columns k1 = 2 m + grp outside the band are zero (Q1 skips them)
       v[i] = centred_abs(2 * (j + i * T) + grp, K) <= A.band ? row[2 * (j + i * T)] : make_float2(0.f, 0.f);
-    split_inverse<LOGK - 1>(v, buf, j, A.tw, A.twp, grp);
-    const float ca = A.cinv[a];
+    split_inverse<LOGK - 1>(v, buf, j, A.tw, A.twp, g4);
+    const float2 ca = A.cinv[a];
     const float2 cha = CH ? A.chirp[a] : make_float2(1.f, 0.f);
-    const float2* be = smem;
-    const float2* bo = smem + Sg::SROW;
-    for (int q = threadIdx.x; q < N; q += 2 * T) {
+    const float2* be = smem + 2 * rr * Sg::SROW;
+    const float2* bo = be + Sg::SROW;
+    for (int q = tr; q < N; q += 2 * T) {
       const int b = q < H ? q + H : q - H;
       const float2 x = split_combine(be[PADI(q)], bo[PADI(q)], q, N, A.tw);
       if (CH) {  // Re{conj(chirp) x}: the adjoint of the centre chirp of Z_s
         const float2 c = cmul(cha, A.chirp[b]);
-        gs[q2 * N + b] = (x.x * c.x + x.y * c.y) * ca * A.cinv[b];
+        gs[q2 * N + b] = correct(x.x * c.x + x.y * c.y, ca, A.cinv[b]);
       } else {
-        gs[q2 * N + b] = x.x * ca * A.cinv[b];
+        gs[q2 * N + b] = correct(x.x, ca, A.cinv[b]);
       }
     }
   }
   __syncthreads();
-  q2_epilogue<CH>(A, gs, a0, threadIdx.x, 2 * T);
+  q2_epilogue<CH>(A, gs, a0, threadIdx.x, R * 2 * T);
 }
 
 // ---------------------------------------------------------------- launchers
@@ -781,7 +796,8 @@ int launch_adjoint_split(pnp_plan* p, const FftArgs& A) {
   constexpr int N = Sg::N, T = Sg::T;
   constexpr int RQ = 4 * T <= 1024 ? 2 : 1;  // grid rows per Q1 CTA (two thread groups each)
   const int smem1 = 2 * RQ * Sg::SROW * 8;
-  const int smem2 = 2 * Sg::SROW * 8 + 2 * N * 4;
+  constexpr int R2 = q2_rows<LOGK>();
+  const int smem2 = 2 * R2 * Sg::SROW * 8 + 2 * N * 4;
   static bool attr = false;
   if (!attr) {
     PNP_CUDA(cudaFuncSetAttribute(fft_q1s<LOGK, RQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem1));
@@ -792,9 +808,9 @@ int launch_adjoint_split(pnp_plan* p, const FftArgs& A) {
   fft_q1s<LOGK, RQ><<<2 * N / RQ, RQ * 2 * T, smem1, p->stream>>>(A);
   PNP_CHECK_LAUNCH();
   if (A.chirp)
-    fft_q2s<LOGK, true><<<N / 2, 2 * T, smem2, p->stream>>>(A);
+    fft_q2s<LOGK, true><<<N / 2, R2 * 2 * T, smem2, p->stream>>>(A);
   else
-    fft_q2s<LOGK, false><<<N / 2, 2 * T, smem2, p->stream>>>(A);
+    fft_q2s<LOGK, false><<<N / 2, R2 * 2 * T, smem2, p->stream>>>(A);
   PNP_CHECK_LAUNCH();
   return PNP_OK;
 }

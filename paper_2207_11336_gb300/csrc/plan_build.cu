@@ -258,8 +258,11 @@ int plan_build(pnp_plan* p, const double* uvw, const int8_t* Jrow, const int32_t
   p->beta = kb_beta(J, (double)K / n);
 
   // grid correction and twiddles
-  std::vector<float> cinv(n);
-  for (int a = 0; a < n; ++a) cinv[a] = (float)(1.0 / kb_correction(a - n / 2, J, p->beta, K));
+  std::vector<float2> cinv(n);
+  for (int a = 0; a < n; ++a) {
+    const double c = 1.0 / kb_correction(a - n / 2, J, p->beta, K);
+    cinv[a] = make_float2((float)c, (float)(c - (double)(float)c));
+  }
   std::vector<float2> tw(K);
   for (int j = 0; j < K; ++j) {
     const double ang = -2.0 * M_PI * j / K;
@@ -468,7 +471,7 @@ int plan_build(pnp_plan* p, const double* uvw, const int8_t* Jrow, const int32_t
     if (int rc = dev_alloc(p, &p->d_gacc, (size_t)n * n)) return rc;
     PNP_CUDA(cudaMemcpy(p->d_chirp, ch.data(), ch.size() * sizeof(float2), cudaMemcpyHostToDevice));
   }
-  PNP_CUDA(cudaMemcpy(p->d_cinv, cinv.data(), n * sizeof(float), cudaMemcpyHostToDevice));
+  PNP_CUDA(cudaMemcpy(p->d_cinv, cinv.data(), n * sizeof(float2), cudaMemcpyHostToDevice));
   PNP_CUDA(cudaMemcpy(p->d_tw, tw.data(), K * sizeof(float2), cudaMemcpyHostToDevice));
   {
     std::vector<float2> twp(TWP_ENTRIES);

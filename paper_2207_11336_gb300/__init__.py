@@ -256,11 +256,11 @@ class Plan:
         _check(lib().pnp_plan_set_compensated(self._h, 1 if enable else 0))
 
     def set_row_batch(self, row_batch: int):
-        """Rows of a run whose residuals one warp forms together (1, 2 or 4)."""
+        """Row batch setting (1, 2 or 4): kept and reported, without an effect on the present kernels."""
         _check(lib().pnp_plan_set_row_batch(self._h, int(row_batch)))
 
     def autotune(self, reps: int = 2) -> dict:
-        """Time the gridding pass's run cap x unit size x row batch candidates and keep the fastest."""
+        """Time the gridding pass's unit sizes and keep the fastest."""
         r, u, ms = C.c_int(), C.c_int64(), C.c_double()
         _check(lib().pnp_plan_autotune(self._h, int(reps), C.byref(r), C.byref(u), C.byref(ms)))
         return {"run_max": r.value, "unit_nnz": u.value, "row_batch": self.info["row_batch"],

@@ -176,6 +176,7 @@ struct pnp_plan {
   // lies in it (the pruned F of Eq. 1: G reads no other cell and writes no other cell).
   int* d_rowh = nullptr;       // K
   int band = -1;
+  bool support_in_l2 = true;   // the gridding pass finds the cells that it adds to in L2 (plan_build)
   int holo_S = 0;
   bool holo = false;           // FB loop and op_norm apply H instead of streaming G
   int64_t device_bytes = 0;

@@ -386,6 +386,13 @@ int plan_build(pnp_plan* p, const double* uvw, const int8_t* Jrow, const int32_t
     p->band = -1;
     for (int k = 0; k < K; ++k)
       if (rowh[k] >= 0) p->band = std::max(p->band, std::abs(centred(k)));
+    int64_t cells = 0;  // of a grid that the FFT passes read and write: the uv support, all of it unless n = K/2
+    for (int k = 0; k < K; ++k) cells += n == K / 2 ? std::clamp(2 * rowh[k] + 1, 0, K) : K;
+    int l2 = 0;
+    PNP_CUDA(cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, p->device));
+    // Adjoint gridding of uniform and track coverage without and with the lines fetched ahead: 16 MB of support 75 and
+    // 55 us (1e6 track rows, J = 7: 92 and 70 us), 41 MB 232 and 89 us; 5 MB 32.4 and 32.8 us.
+    p->support_in_l2 = cells * (int64_t)sizeof(float2) <= l2 / 16;
   }
   std::vector<RowGeom>().swap(geom);
 

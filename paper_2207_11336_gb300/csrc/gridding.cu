@@ -51,11 +51,11 @@ constexpr int RING = 4;  // rows of each lane group's ring
 struct GArgs {
   int K, logK, ntc;             // grid side, log2 K, tiles per side
   const Unit* units;
-  long long u_begin, n_units;   // this launch walks units [u_begin, n_units) (one w-stack and class)
+  unsigned u_begin, n_units;    // this launch walks units [u_begin, n_units) (one w-stack and class)
   const unsigned char* rows;    // stored rows (row_units(J) 16-byte units each)
   const int* rowh;              // uv support: per grid row the largest centred |k0| of a tap (-1: none)
-  unsigned* sched;              // [0] next batch of units, [1] warps done; both zero between launches
-  int batch;                    // units per batch
+  unsigned* sched;              // [0] batches taken, [1] warps done; both zero between launches.  NULL: a batch per warp
+  unsigned batch;               // units per batch
   int prefetch;                 // the cells of gridB that taps reach do not stay in L2
   const int32_t* perm;
   const float2* y_in;   // sorted order (G_GRID, G_FUSED); NULL in G_FUSED = no data term
@@ -129,23 +129,68 @@ __device__ __forceinline__ void group_sum(float& re, float& im, int lane) {
   im = up ? v : w;
 }
 
-// Adds one cell of a unit's accumulator to the output grid.  Compensated: the atomic returns the value
-// it added to, so the lane forms the exact rounding error of the (round-to-nearest) sum (TwoSum) and adds
-// it to the compensation grid.
-__device__ __forceinline__ void flush_cell(const GArgs& A, float2 v, int k1, int k0) {
-  if (v.x == 0.f && v.y == 0.f) return;
-  // The padding tap rows of a window hold exact zeros unless a visibility is not finite; the NaN they hold
-  // then must not reach a cell outside the uv support, which nothing zeroes again.
-  if (!(v.x == v.x && v.y == v.y) && min(k0, A.K - k0) > A.rowh[k1]) return;
-  const size_t g = ((size_t)k1 << A.logK) + k0;
-  if (!A.gridB_lo) {
-    atomicAdd(&A.gridB[g], v);
+// Whether a cell of an accumulator goes to the output grid.  The padding tap rows of a window hold exact zeros
+// unless a visibility is not finite; the NaN they hold then must not reach a cell outside the uv support, which
+// nothing zeroes again.
+__device__ __forceinline__ bool flushed(const GArgs& A, float2 v, int k1, int k0) {
+  return !(v.x == 0.f && v.y == 0.f) && ((v.x == v.x && v.y == v.y) || min(k0, A.K - k0) <= A.rowh[k1]);
+}
+
+// Compensated flush of a region: the atomic returns the value it added to, so the lane forms the exact rounding error
+// of the (round-to-nearest) sum (TwoSum) and adds it to the compensation grid; the atomics of FB row pairs are in flight
+// together.  Out of line, so that its registers do not count against the main loop.
+template <int PR, int NC, int RL>
+__device__ __noinline__ void flush_compensated(const GArgs& A, ulonglong2* sy, int r0, int c0, int lane) {
+  constexpr int RI = 32 / RL, FB = 3;
+  const int Km = A.K - 1, jc = lane % RL, gc = (c0 + jc) & Km;
+  if (jc >= NC) return;
+  for (int i0 = lane / RL; i0 < PR; i0 += FB * RI) {
+    float2 v[2 * FB], old[2 * FB];
+    bool on[2 * FB];
+#pragma unroll
+    for (int f = 0; f < 2 * FB; ++f) {
+      const int i = i0 + (f >> 1) * RI, k1 = (r0 + 2 * i + (f & 1)) & Km;
+      on[f] = false;
+      if (i < PR) {
+        const float4 q = *reinterpret_cast<const float4*>(&sy[i * NC + jc]);
+        v[f] = f & 1 ? make_float2(q.y, q.w) : make_float2(q.x, q.z);
+        if (f & 1) sy[i * NC + jc] = make_ulonglong2(0, 0);
+        on[f] = flushed(A, v[f], k1, gc);
+        if (on[f]) old[f] = atomicAdd(&A.gridB[((size_t)k1 << A.logK) + gc], v[f]);
+      }
+    }
+#pragma unroll
+    for (int f = 0; f < 2 * FB; ++f) {
+      if (!on[f]) continue;
+      const size_t g = ((size_t)((r0 + 2 * (i0 + (f >> 1) * RI) + (f & 1)) & Km) << A.logK) + gc;
+      const float ex = two_sum_err(old[f].x, v[f].x, __fadd_rn(old[f].x, v[f].x));
+      const float ey = two_sum_err(old[f].y, v[f].y, __fadd_rn(old[f].y, v[f].y));
+      if (ex != 0.f || ey != 0.f) atomicAdd(&A.gridB_lo[g], __floats2bfloat162_rn(ex, ey));
+    }
+  }
+}
+
+// Adds a warp's accumulator (the region from grid row r0 and column c0 on) to the output grid and clears it.
+template <typename L, bool COMP>
+__device__ __forceinline__ void flush_region(const GArgs& A, ulonglong2* sy, int r0, int c0, int lane) {
+  constexpr int NC = L::NC, RL = L::RL, RI = 32 / RL;
+  if constexpr (COMP) {
+    flush_compensated<L::PR, NC, RL>(A, sy, r0, c0, lane);
     return;
   }
-  const float2 old = atomicAdd(&A.gridB[g], v);
-  const float ex = two_sum_err(old.x, v.x, __fadd_rn(old.x, v.x));
-  const float ey = two_sum_err(old.y, v.y, __fadd_rn(old.y, v.y));
-  if (ex != 0.f || ey != 0.f) atomicAdd(&A.gridB_lo[g], __floats2bfloat162_rn(ex, ey));
+  const int Km = A.K - 1, jc = lane % RL, gc = (c0 + jc) & Km;
+  if (jc >= NC) return;
+#pragma unroll 2
+  for (int i = lane / RL; i < L::PR; i += RI) {
+    const float4 v = *reinterpret_cast<const float4*>(&sy[i * NC + jc]);
+    sy[i * NC + jc] = make_ulonglong2(0, 0);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const float2 c = h ? make_float2(v.y, v.w) : make_float2(v.x, v.z);
+      const int k1 = (r0 + 2 * i + h) & Km;
+      if (flushed(A, c, k1, gc)) atomicAdd(&A.gridB[((size_t)k1 << A.logK) + gc], c);
+    }
+  }
 }
 
 // shared memory of one warp: the groups' rings of rows and of visibilities (or output positions), the
@@ -156,6 +201,7 @@ struct Layout {
   static constexpr int UNITS = BF ? JP * JP : 2 * JP, RBYTES = 16 * UNITS;
   static constexpr int Q = tap_quant(JP, W);  // first-tap columns of a window
   static constexpr int PR = GT / 2 - 1 + JP, NC = GT - Q + W, CELLS = PR * NC;
+  static constexpr int RL = NC <= 16 ? 16 : 32;  // lanes on a row pair of a region
   static constexpr int YR = NG * RING * RBYTES, YB = NG * RING * 8;
   static constexpr int OUT = YR + YB, IN = OUT + (MODE == G_DEGRID ? 0 : CELLS * 16);
   static constexpr int BYTES = (IN + (MODE == G_GRID ? 0 : CELLS * 16) + 127) & ~127;
@@ -167,7 +213,8 @@ constexpr int min_ctas() {
   return JP <= 6 ? 5 : 4;
 }
 
-template <int MODE, bool BF, int JP, int W>
+// COMP: the flushes are compensated
+template <int MODE, bool BF, int JP, int W, bool COMP>
 __global__ void __launch_bounds__(GPASS_WARPS * 32, min_ctas<JP>()) gpass(const __grid_constant__ GArgs A) {
   using L = Layout<MODE, BF, JP, W>;
   constexpr int NG = L::NG, NC = L::NC, Q = L::Q;
@@ -188,13 +235,12 @@ __global__ void __launch_bounds__(GPASS_WARPS * 32, min_ctas<JP>()) gpass(const 
   if (MODE != G_DEGRID)
     for (int c = lane; c < L::CELLS; c += 32) sy[c] = zero4;
   const uint32_t ring_a = smem_u32(ring) + li * 16, yring_a = smem_u32(yring);
-  unsigned nb = 0;
-  if (lane == 0) nb = atomicAdd(A.sched, 1u);
-  nb = __shfl_sync(0xffffffffu, nb, 0);
-  long long u = A.u_begin + (long long)nb * A.batch;
+  const unsigned warps = gridDim.x * GPASS_WARPS;
+  unsigned nb = blockIdx.x * GPASS_WARPS + (threadIdx.x >> 5);  // the first batch; the others from the counter
+  unsigned u = A.u_begin + nb * A.batch;  // units are no more than rows: the sums stay below 2^32
   while (u < A.n_units) {
-    const long long ue = min(u + A.batch, A.n_units);
-    if (lane == 0) nb = atomicAdd(A.sched, 1u);  // the next batch, known by the end of this one
+    const unsigned ue = min(u + A.batch, A.n_units);
+    if (lane == 0 && A.sched) nb = warps + atomicAdd(A.sched, 1u);  // the next batch, known by the end of this one
     for (; u < ue; ++u) {
       const Unit U = A.units[u];
       const int t1 = U.tile / A.ntc, t0 = U.tile - t1 * A.ntc;
@@ -237,9 +283,9 @@ __global__ void __launch_bounds__(GPASS_WARPS * 32, min_ctas<JP>()) gpass(const 
 #pragma unroll
       for (int s = 0; s < RING - 1; ++s) fetch(s);
       // this lane's column of the regions (two row pairs at a time where 16 lanes hold a row)
-      constexpr int RL = NC <= 16 ? 16 : 32, RI = 32 / RL;
-      const int jc = lane % RL, ri = lane / RL, gc = (c0 + jc) & Km;
+      constexpr int RL = L::RL, RI = 32 / RL;
       if (MODE != G_GRID) {
+        const int jc = lane % RL, ri = lane / RL, gc = (c0 + jc) & Km;
         if (jc < NC) {
 #pragma unroll 3
           for (int i = ri; i < L::PR; i += RI) {
@@ -356,24 +402,17 @@ __global__ void __launch_bounds__(GPASS_WARPS * 32, min_ctas<JP>()) gpass(const 
       }
       if (MODE != G_DEGRID) {
         retire(0xffffffffu);
-        if (jc < NC) {
-#pragma unroll 2
-          for (int i = ri; i < L::PR; i += RI) {
-            const float4 v = *reinterpret_cast<const float4*>(&sy[i * NC + jc]);
-            sy[i * NC + jc] = zero4;
-            flush_cell(A, make_float2(v.x, v.z), (r0 + 2 * i) & Km, gc);
-            flush_cell(A, make_float2(v.y, v.w), (r0 + 2 * i + 1) & Km, gc);
-          }
-        }
+        flush_region<L, COMP>(A, sy, r0, c0, lane);
       }
     }
+    if (!A.sched) break;
     nb = __shfl_sync(0xffffffffu, nb, 0);
-    u = A.u_begin + (long long)nb * A.batch;
+    u = A.u_begin + nb * A.batch;
   }
   // This kernel ends only after the previous class's kernel has (when it was launched as its dependent), so that
   // the end of the last class's kernel is the end of the pass.
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  if (lane == 0 && atomicAdd(A.sched + 1, 1u) == gridDim.x * GPASS_WARPS - 1) {  // the last warp: every batch is taken
+  if (lane == 0 && A.sched && atomicAdd(A.sched + 1, 1u) == warps - 1) {  // the last warp: every batch is taken
     A.sched[0] = 0;
     A.sched[1] = 0;
   }
@@ -390,24 +429,25 @@ __global__ void permute_kernel(const float2* __restrict__ y, const int32_t* __re
 
 // The classes' kernels of one pass only add to the grid (or write their own rows), so each after the first is launched
 // as a programmatic dependent of the one before: its CTAs fill the tail of that kernel instead of waiting for its end.
-template <int MODE, bool BF, int JP, int W>
+template <int MODE, bool BF, int JP, int W, bool COMP>
 int launch_class(pnp_plan* p, GArgs A, int s, bool* first) {
   const int c = s * TAP_CLASSES + tap_class(JP, W);
-  A.u_begin = p->h_class_units[c];
-  A.n_units = p->h_class_units[c + 1];
-  const long long count = A.n_units - A.u_begin;
+  A.u_begin = (unsigned)p->h_class_units[c];
+  A.n_units = (unsigned)p->h_class_units[c + 1];
+  const long long count = (long long)A.n_units - A.u_begin;
   if (count <= 0) return PNP_OK;
   const int smem = GPASS_WARPS * Layout<MODE, BF, JP, W>::BYTES;
   static int per_sm = 0;
   if (per_sm == 0) {
-    PNP_CUDA(cudaFuncSetAttribute(gpass<MODE, BF, JP, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    PNP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, gpass<MODE, BF, JP, W>, GPASS_WARPS * 32, smem));
+    PNP_CUDA(cudaFuncSetAttribute(gpass<MODE, BF, JP, W, COMP>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    PNP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, gpass<MODE, BF, JP, W, COMP>, GPASS_WARPS * 32, smem));
     if (per_sm < 1) return fail(PNP_ERR_UNSUPPORTED, "gridding regions do not fit in shared memory");
   }
   const long long grid = std::min((long long)per_sm * p->num_sms, (count + GPASS_WARPS - 1) / GPASS_WARPS);
   // about 16 batches per warp: the counter is taken seldom, the last batches are short
-  A.batch = (int)std::max(1ll, std::min(16ll, count / (grid * GPASS_WARPS * 16)));
-  A.sched = p->d_sched + 2 * c;
+  A.batch = (unsigned)std::max(1ll, std::min(16ll, count / (grid * GPASS_WARPS * 16)));
+  // one batch per warp needs no counter (3 of 10 us where the whole pass is one unit per warp)
+  A.sched = count > grid * GPASS_WARPS * A.batch ? p->d_sched + 2 * c : nullptr;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)grid);
   cfg.blockDim = dim3(GPASS_WARPS * 32);
@@ -419,26 +459,32 @@ int launch_class(pnp_plan* p, GArgs A, int s, bool* first) {
   cfg.attrs = &at;
   cfg.numAttrs = *first ? 0 : 1;
   *first = false;
-  PNP_CUDA(cudaLaunchKernelEx(&cfg, gpass<MODE, BF, JP, W>, A));
+  PNP_CUDA(cudaLaunchKernelEx(&cfg, gpass<MODE, BF, JP, W, COMP>, A));
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return PNP_OK;
 }
 
-template <int MODE, bool BF>
+template <int MODE, bool BF, bool COMP>
 int launch_classes(pnp_plan* p, const GArgs& A, int s) {
-  bool first = true;  // the largest supports first: the short classes fill the tails
-  if (int rc = launch_class<MODE, BF, 9, 16>(p, A, s, &first)) return rc;
-  if (int rc = launch_class<MODE, BF, 8, 16>(p, A, s, &first)) return rc;
-  if (int rc = launch_class<MODE, BF, 7, 16>(p, A, s, &first)) return rc;
-  if (int rc = launch_class<MODE, BF, 6, 16>(p, A, s, &first)) return rc;
-  if (int rc = launch_class<MODE, BF, 5, 16>(p, A, s, &first)) return rc;
-  if (int rc = launch_class<MODE, BF, 5, 8>(p, A, s, &first)) return rc;
-  return launch_class<MODE, BF, 4, 8>(p, A, s, &first);
+  bool first = true;
+  // the largest supports first: the short classes fill the tails
+  if (int rc = launch_class<MODE, BF, 9, 16, COMP>(p, A, s, &first)) return rc;
+  if (int rc = launch_class<MODE, BF, 8, 16, COMP>(p, A, s, &first)) return rc;
+  if (int rc = launch_class<MODE, BF, 7, 16, COMP>(p, A, s, &first)) return rc;
+  if (int rc = launch_class<MODE, BF, 6, 16, COMP>(p, A, s, &first)) return rc;
+  if (int rc = launch_class<MODE, BF, 5, 16, COMP>(p, A, s, &first)) return rc;
+  if (int rc = launch_class<MODE, BF, 5, 8, COMP>(p, A, s, &first)) return rc;
+  return launch_class<MODE, BF, 4, 8, COMP>(p, A, s, &first);
 }
 
 template <int MODE>
 int dispatch(pnp_plan* p, const GArgs& A, int s) {
-  return p->wdtype == PNP_W_BF16C ? launch_classes<MODE, true>(p, A, s) : launch_classes<MODE, false>(p, A, s);
+  const bool bf = p->wdtype == PNP_W_BF16C;
+  if (MODE != G_DEGRID && A.gridB_lo) {
+    constexpr bool C = MODE != G_DEGRID;
+    return bf ? launch_classes<MODE, true, C>(p, A, s) : launch_classes<MODE, false, C>(p, A, s);
+  }
+  return bf ? launch_classes<MODE, true, false>(p, A, s) : launch_classes<MODE, false, false>(p, A, s);
 }
 
 }  // namespace

@@ -54,7 +54,7 @@ __host__ __device__ __forceinline__ float2 cmulc(float2 a, float2 b) {
 // taps lie in one GT x GT grid tile (and one data block): the work of one warp.
 constexpr int GT = 8;               // gridding tile side (first-tap cells)
 constexpr int GKT = 32;             // side of the coarse tiles of the (tile, block) sort key
-constexpr int GPASS_WARPS = 4;      // warps per gridding CTA (they work independently)
+constexpr int MIX_TILE = 16;        // tile side of a plan with thin units (pick_tile in plan_build.cu)
 constexpr int TAP_CLASSES = 7;      // classes of supports: J <= 7, 8, 9, 11, 13, 15, 16 (tap_class)
 // twiddles of the radix-16 passes 1 and 2 of the FFT: entry off(p) + r 16^p + k holds
 // exp(-2 pi i r k / 16^(p+1)), off(1) = 0, off(2) = 256 (independent of the transform length)
@@ -66,7 +66,7 @@ constexpr int TWP_ENTRIES = 16 * 16 + 16 * 256;
 //              the k0 axis: 2 tap_pairs 16-byte units;
 //   BF16:      the rounded taps [k1 pair][k0](re, re, im, im): tap_pairs^2 16-byte units.
 // The last k0 entry is never a tap (2 tap_pairs > J): it holds the first tap's cell in the tile,
-// row << 3 | column (BF16: that of pair 0), at byte row_cell_at.
+// coarse row << 5 | coarse column within its GKT x GKT coarse tile (BF16: that of pair 0), at byte row_cell_at.
 __host__ __device__ constexpr int tap_pairs(int J) { return J <= 7 ? 4 : (J + 2) / 2; }
 __host__ __device__ constexpr int tap_lanes(int J) { return J <= 8 ? 8 : 16; }  // lanes that share a row
 __host__ __device__ constexpr int tap_class(int pairs, int lanes) { return pairs == 4 ? 0 : lanes == 8 ? 1 : pairs - 3; }
@@ -87,7 +87,7 @@ __device__ __forceinline__ int row_cell(const unsigned char* row, int J, bool bf
 // tap (i1, i0) of a stored row with support J (i0, i1 < J)
 __device__ __forceinline__ float2 row_tap(const unsigned char* row, int J, bool bf16, int i1, int i0) {
   const int jp = tap_pairs(J);
-  i1 += (row_cell(row, J, bf16) >> 3) & 1;
+  i1 += (row_cell(row, J, bf16) >> 5) & 1;
   if (bf16) {
     const __nv_bfloat16* o = reinterpret_cast<const __nv_bfloat16*>(row) + ((i1 >> 1) * 2 * jp + i0) * 4 + (i1 & 1);
     return make_float2(__bfloat162float(o[0]), __bfloat162float(o[2]));
@@ -102,8 +102,8 @@ struct Unit {
   long long row_unit;   // its offset in the stored rows, 16-byte units
   int nrows;
   int J;
-  int tile;             // t1 * (K / GT) + t0
-  int pad_;
+  int tile;             // t1 * (K / tile side) + t0
+  int first;            // 1: starts a tile's units (or a piece of a large tile); 0: goes on with the unit before's regions
 };
 constexpr int RUN_MAX = 6;  // reported default of the run cap setting
 
@@ -120,6 +120,7 @@ enum GMode { G_DEGRID = 0, G_GRID = 1, G_FUSED = 2 };
 struct pnp_plan {
   int n = 0, K = 0, logK = 0, J = 7, Jmax = 7, wdtype = PNP_W_C64, nblocks = 1;
   int tile = pnp::GT;  // gridding tile side (cells)
+  bool mixed = false;  // thin units: one kernel for all supports (pick_tile)
   int ntc = 0;         // tiles per grid side, K / tile
   int pitch = 0;       // side and row pitch (cells) of a warp's gridding regions
   int run_max = pnp::RUN_MAX, row_batch = 2;  // settings without an effect on the present kernels (reported)

@@ -29,7 +29,9 @@
 // one 16-byte access per pair of taps.
 // The rows stream through a per-warp ring of cp.async copies.
 //
-// The rows of each class of supports run as a kernel of their own: its registers and
+// Where rows are so sparse that the units hold one or two (pick_tile in plan_build.cu), larger tiles are taken and
+// one kernel walks the units of all supports of a tile with the same regions.
+// Elsewhere the rows of each class of supports run as a kernel of their own: its registers and
 // regions are sized for that class, and all warps of an SM execute the same code (one
 // kernel for every class spent 42% of its warp time on instruction fetches).  Warps take
 // batches of units from a counter.
@@ -45,8 +47,6 @@
 
 namespace pnp {
 namespace {
-
-constexpr int RING = 4;  // rows of each lane group's ring
 
 struct GArgs {
   int K, logK, ntc;             // grid side, log2 K, tiles per side
@@ -195,29 +195,34 @@ __device__ __forceinline__ void flush_region(const GArgs& A, ulonglong2* sy, int
 
 // shared memory of one warp: the groups' rings of rows and of visibilities (or output positions), the
 // accumulator region and the input region, both PR pairs of grid rows by NC columns of (re, re, im, im)
-template <int MODE, bool BF, int JP, int W_>
+template <int MODE, bool BF, int JP, int W_, bool MIX>
 struct Layout {
+  static constexpr int WARPS = MIX ? 2 : 4;  // per CTA (they work independently)
+  static constexpr int RING = MIX && BF ? 2 : 4;  // rows of each lane group's ring
   static constexpr int W = W_, NG = 32 / W;
-  static constexpr int UNITS = BF ? JP * JP : 2 * JP, RBYTES = 16 * UNITS;
-  static constexpr int Q = tap_quant(JP, W);  // first-tap columns of a window
-  static constexpr int PR = GT / 2 - 1 + JP, NC = GT - Q + W, CELLS = PR * NC;
-  static constexpr int RL = NC <= 16 ? 16 : 32;  // lanes on a row pair of a region
+  static constexpr int UNITS = BF ? JP * JP : 2 * JP, RBYTES = 16 * UNITS;  // of the largest support
+  static constexpr int T = MIX ? MIX_TILE : GT;           // tile side
+  static constexpr int Q = MIX ? 1 : tap_quant(JP, W);    // first-tap columns of a window
+  static constexpr int PR = T / 2 - 1 + JP, NC = T - Q + W, CELLS = PR * NC;
+  static constexpr int RL = NC <= 16 ? 16 : 32;           // lanes on a row pair of a region
   static constexpr int YR = NG * RING * RBYTES, YB = NG * RING * 8;
   static constexpr int OUT = YR + YB, IN = OUT + (MODE == G_DEGRID ? 0 : CELLS * 16);
   static constexpr int BYTES = (IN + (MODE == G_GRID ? 0 : CELLS * 16) + 127) & ~127;
 };
 
 // resident CTAs the registers allow for, per class
-template <int JP>
+template <int JP, bool MIX>
 constexpr int min_ctas() {
-  return JP <= 6 ? 5 : 4;
+  return MIX ? (JP <= 6 ? 8 : 6) : JP <= 6 ? 5 : 4;
 }
 
-// COMP: the flushes are compensated
-template <int MODE, bool BF, int JP, int W, bool COMP>
-__global__ void __launch_bounds__(GPASS_WARPS * 32, min_ctas<JP>()) gpass(const __grid_constant__ GArgs A) {
-  using L = Layout<MODE, BF, JP, W>;
-  constexpr int NG = L::NG, NC = L::NC, Q = L::Q;
+// MIX: the units of a plan whose units are thin (pick_tile), of any support with tap_pairs <= JP; the regions are kept
+// from one unit of a tile to the next.  Otherwise the units hold rows of the class of supports (JP, W).  COMP: the flushes
+// are compensated.
+template <int MODE, bool BF, int JP, int W, bool MIX, bool COMP>
+__global__ void __launch_bounds__(32 * Layout<MODE, BF, JP, W, MIX>::WARPS, min_ctas<JP, MIX>()) gpass(const __grid_constant__ GArgs A) {
+  using L = Layout<MODE, BF, JP, W, MIX>;
+  constexpr int NG = L::NG, NC = L::NC, Q = L::Q, T = L::T, RING = L::RING;
   extern __shared__ __align__(128) unsigned char sm[];
   const int lane = threadIdx.x & 31;
   const int gi = lane / W, li = lane % W;
@@ -235,23 +240,33 @@ __global__ void __launch_bounds__(GPASS_WARPS * 32, min_ctas<JP>()) gpass(const 
   if (MODE != G_DEGRID)
     for (int c = lane; c < L::CELLS; c += 32) sy[c] = zero4;
   const uint32_t ring_a = smem_u32(ring) + li * 16, yring_a = smem_u32(yring);
-  const unsigned warps = gridDim.x * GPASS_WARPS;
-  unsigned nb = blockIdx.x * GPASS_WARPS + (threadIdx.x >> 5);  // the first batch; the others from the counter
+  const unsigned warps = gridDim.x * L::WARPS;
+  unsigned nb = blockIdx.x * L::WARPS + (threadIdx.x >> 5);  // the first batch; the others from the counter
   unsigned u = A.u_begin + nb * A.batch;  // units are no more than rows: the sums stay below 2^32
   while (u < A.n_units) {
     const unsigned ue = min(u + A.batch, A.n_units);
     if (lane == 0 && A.sched) nb = warps + atomicAdd(A.sched, 1u);  // the next batch, known by the end of this one
-    for (; u < ue; ++u) {
+    int held = -1;  // MIX: the tile whose regions are staged
+    for (; u < (MIX ? A.n_units : ue); ++u) {
       const Unit U = A.units[u];
+      if (MIX) {  // a batch is the tiles that start in it
+        if (U.first && u >= ue) break;
+        if (!U.first && held < 0) continue;
+        if (MODE != G_DEGRID && U.first && held >= 0)
+          flush_region<L, COMP>(A, sy, held / A.ntc * T, held % A.ntc * T, lane);
+      }
       const int t1 = U.tile / A.ntc, t0 = U.tile - t1 * A.ntc;
-      const int r0 = t1 * GT, c0 = t0 * GT, J = U.J;
-      if (J < 2 || tap_pairs(J) != JP || tap_lanes(J) != W) {
+      const int r0 = t1 * T, c0 = t0 * T, J = U.J;
+      const bool fresh = !MIX || U.first;
+      if (MIX) held = U.tile;
+      if (J < 2 || (MIX ? tap_pairs(J) > JP : tap_pairs(J) != JP || tap_lanes(J) != W)) {
         if (lane == 0) atomicOr(A.status, 4);  // inconsistent work list: skip the unit
         continue;
       }
+      const int jp = MIX ? tap_pairs(J) : JP, units = MIX ? row_units(J, BF) : L::UNITS;
       const int n = (U.nrows + NG - 1) / NG;  // steps; rows of this group:
       const int q0 = min(gi * n, U.nrows), mine = min(n, U.nrows - q0);
-      const unsigned char* src = A.rows + ((size_t)U.row_unit << 4) + (size_t)q0 * L::RBYTES + li * 16;
+      const unsigned char* src = A.rows + ((size_t)U.row_unit << 4) + (size_t)q0 * (16 * units) + li * 16;
       const int32_t* psrc = A.perm + U.row_begin + q0;
       const float2* ysrc = A.y_in + U.row_begin + q0;
       const bool has_y = A.y_in != nullptr;
@@ -260,8 +275,8 @@ __global__ void __launch_bounds__(GPASS_WARPS * 32, min_ctas<JP>()) gpass(const 
           const uint32_t slot = s % RING;
 #pragma unroll
           for (int c = 0; c < L::UNITS; c += W)
-            if (c + W <= L::UNITS || c + li < L::UNITS) cp16(ring_a + slot * L::RBYTES + c * 16, src + c * 16);
-          src += L::RBYTES;
+            if ((!MIX && c + W <= L::UNITS) || c + li < units) cp16(ring_a + slot * L::RBYTES + c * 16, src + c * 16);
+          src += 16 * units;
           if (li == 0) {
             if (MODE == G_DEGRID) cp4(yring_a + slot * 8, psrc);
             else if (has_y) cp8(yring_a + slot * 8, ysrc);
@@ -274,7 +289,7 @@ __global__ void __launch_bounds__(GPASS_WARPS * 32, min_ctas<JP>()) gpass(const 
       // Atomics on lines that are not in L2 are served far below the rate of plain fetches, so the lines that the
       // unit's flush will add to are fetched ahead (adjoint of 3e5 J = 7 rows spread over a 4096^2 grid: 285 -> 128 us,
       // 1e6 rows of J 7-16: 1050 -> 595 us).
-      if (MODE != G_DEGRID && A.prefetch && lane < 2 * L::PR) {
+      if (MODE != G_DEGRID && A.prefetch && fresh && lane < 2 * L::PR) {
         const float2* g = A.gridB + ((size_t)((r0 + lane) & Km) << A.logK);
 #pragma unroll
         for (int c = 0; c < NC; c += 8) asm volatile("prefetch.global.L2 [%0];" ::"l"(g + ((c0 + c) & Km)));
@@ -286,7 +301,7 @@ __global__ void __launch_bounds__(GPASS_WARPS * 32, min_ctas<JP>()) gpass(const 
       constexpr int RL = L::RL, RI = 32 / RL;
       if (MODE != G_GRID) {
         const int jc = lane % RL, ri = lane / RL, gc = (c0 + jc) & Km;
-        if (jc < NC) {
+        if (fresh && jc < NC) {
 #pragma unroll 3
           for (int i = ri; i < L::PR; i += RI) {
             const float2 a = A.gridA[((size_t)((r0 + 2 * i) & Km) << A.logK) + gc];
@@ -324,7 +339,8 @@ __global__ void __launch_bounds__(GPASS_WARPS * 32, min_ctas<JP>()) gpass(const 
         const unsigned char* rp = ring + (s % RING) * L::RBYTES;
         const unsigned char* yp = yring + (s % RING) * 8;
         const bool act = s < mine;
-        const int cell = *reinterpret_cast<const int*>(rp + row_cell_at(JP, BF)), nw = cell & (0x30 | (7 & ~(Q - 1)));
+        const int cell = *reinterpret_cast<const int*>(rp + row_cell_at(jp, BF)) & ((T - 1) * 33);
+        const int nw = cell & ((T - 2) << 5 | (T - Q));  // row pair and window columns of the first tap
         const int i0 = li - (cell & (Q - 1));            // this lane's tap column of the row
         const bool tap = (unsigned)i0 < (unsigned)J;
         const bool moved = act && nw != win;
@@ -333,7 +349,7 @@ __global__ void __launch_bounds__(GPASS_WARPS * 32, min_ctas<JP>()) gpass(const 
           if (MODE != G_DEGRID) retire(who);
           if (moved) {
             win = nw;
-            base = (nw >> 4) * NC + (nw & 7) + li;
+            base = (nw >> 6) * NC + (nw & 31) + li;
 #pragma unroll
             for (int p = 0; p < JP; ++p) {
               if (MODE != G_GRID) {
@@ -347,11 +363,11 @@ __global__ void __launch_bounds__(GPASS_WARPS * 32, min_ctas<JP>()) gpass(const 
         }
         float2 g0 = make_float2(0.f, 0.f);
         if constexpr (!BF) {
-          if (tap) g0 = reinterpret_cast<const float2*>(rp + 16 * JP)[i0];
+          if (tap) g0 = reinterpret_cast<const float2*>(rp + 16 * jp)[i0];
         }
         auto pair = [&](int p, f2& gx, f2& gy) {  // weights of tap rows 2 p and 2 p + 1
           if constexpr (BF) {
-            const uint2 w = reinterpret_cast<const uint2*>(rp)[p * 2 * JP + (tap ? i0 : 0)];
+            const uint2 w = reinterpret_cast<const uint2*>(rp)[p * 2 * jp + (tap ? i0 : 0)];
             gx = bf2(w.x);
             gy = bf2(w.y);
           } else {
@@ -365,6 +381,7 @@ __global__ void __launch_bounds__(GPASS_WARPS * 32, min_ctas<JP>()) gpass(const 
           f2 a0 = 0, a1 = 0, a2 = 0, a3 = 0;
 #pragma unroll
           for (int p = 0; p < JP; ++p) {
+            if (MIX && p >= jp) break;
             f2 gx, gy;
             pair(p, gx, gy);
             a0 = fma2(gx, xr[p], a0);
@@ -392,6 +409,7 @@ __global__ void __launch_bounds__(GPASS_WARPS * 32, min_ctas<JP>()) gpass(const 
           const f2 tx = pk(r.x, r.x), ty = pk(r.y, r.y), nx = pk(-r.x, -r.x);
 #pragma unroll
           for (int p = 0; p < JP; ++p) {
+            if (MIX && p >= jp) break;
             f2 gx, gy;
             pair(p, gx, gy);
             sr[p] = fma2(gx, tx, fma2(gy, ty, sr[p]));  // += conj(g1) t
@@ -402,9 +420,10 @@ __global__ void __launch_bounds__(GPASS_WARPS * 32, min_ctas<JP>()) gpass(const 
       }
       if (MODE != G_DEGRID) {
         retire(0xffffffffu);
-        flush_region<L, COMP>(A, sy, r0, c0, lane);
+        if (!MIX) flush_region<L, COMP>(A, sy, r0, c0, lane);
       }
     }
+    if (MIX && MODE != G_DEGRID && held >= 0) flush_region<L, COMP>(A, sy, held / A.ntc * T, held % A.ntc * T, lane);
     if (!A.sched) break;
     nb = __shfl_sync(0xffffffffu, nb, 0);
     u = A.u_begin + nb * A.batch;
@@ -429,28 +448,30 @@ __global__ void permute_kernel(const float2* __restrict__ y, const int32_t* __re
 
 // The classes' kernels of one pass only add to the grid (or write their own rows), so each after the first is launched
 // as a programmatic dependent of the one before: its CTAs fill the tail of that kernel instead of waiting for its end.
-template <int MODE, bool BF, int JP, int W, bool COMP>
+template <int MODE, bool BF, int JP, int W, bool MIX, bool COMP>
 int launch_class(pnp_plan* p, GArgs A, int s, bool* first) {
-  const int c = s * TAP_CLASSES + tap_class(JP, W);
+  using L = Layout<MODE, BF, JP, W, MIX>;
+  const int c = s * TAP_CLASSES + (MIX ? 0 : tap_class(JP, W));
   A.u_begin = (unsigned)p->h_class_units[c];
   A.n_units = (unsigned)p->h_class_units[c + 1];
   const long long count = (long long)A.n_units - A.u_begin;
   if (count <= 0) return PNP_OK;
-  const int smem = GPASS_WARPS * Layout<MODE, BF, JP, W>::BYTES;
+  const int smem = L::WARPS * L::BYTES;
   static int per_sm = 0;
+  auto kernel = gpass<MODE, BF, JP, W, MIX, COMP>;
   if (per_sm == 0) {
-    PNP_CUDA(cudaFuncSetAttribute(gpass<MODE, BF, JP, W, COMP>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    PNP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, gpass<MODE, BF, JP, W, COMP>, GPASS_WARPS * 32, smem));
+    PNP_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    PNP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, L::WARPS * 32, smem));
     if (per_sm < 1) return fail(PNP_ERR_UNSUPPORTED, "gridding regions do not fit in shared memory");
   }
-  const long long grid = std::min((long long)per_sm * p->num_sms, (count + GPASS_WARPS - 1) / GPASS_WARPS);
+  const long long grid = std::min((long long)per_sm * p->num_sms, (count + L::WARPS - 1) / L::WARPS);
   // about 16 batches per warp: the counter is taken seldom, the last batches are short
-  A.batch = (unsigned)std::max(1ll, std::min(16ll, count / (grid * GPASS_WARPS * 16)));
+  A.batch = (unsigned)std::max(1ll, std::min(16ll, count / (grid * L::WARPS * 16)));
   // one batch per warp needs no counter (3 of 10 us where the whole pass is one unit per warp)
-  A.sched = count > grid * GPASS_WARPS * A.batch ? p->d_sched + 2 * c : nullptr;
+  A.sched = count > grid * L::WARPS * A.batch ? p->d_sched + 2 * c : nullptr;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3(GPASS_WARPS * 32);
+  cfg.blockDim = dim3(L::WARPS * 32);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = p->stream;
   cudaLaunchAttribute at{};
@@ -459,7 +480,7 @@ int launch_class(pnp_plan* p, GArgs A, int s, bool* first) {
   cfg.attrs = &at;
   cfg.numAttrs = *first ? 0 : 1;
   *first = false;
-  PNP_CUDA(cudaLaunchKernelEx(&cfg, gpass<MODE, BF, JP, W, COMP>, A));
+  PNP_CUDA(cudaLaunchKernelEx(&cfg, kernel, A));
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return PNP_OK;
 }
@@ -467,14 +488,17 @@ int launch_class(pnp_plan* p, GArgs A, int s, bool* first) {
 template <int MODE, bool BF, bool COMP>
 int launch_classes(pnp_plan* p, const GArgs& A, int s) {
   bool first = true;
+  if (p->mixed)
+    return tap_pairs(p->Jmax) <= 5 ? launch_class<MODE, BF, 5, 16, true, COMP>(p, A, s, &first)
+                                   : launch_class<MODE, BF, 9, 16, true, COMP>(p, A, s, &first);
   // the largest supports first: the short classes fill the tails
-  if (int rc = launch_class<MODE, BF, 9, 16, COMP>(p, A, s, &first)) return rc;
-  if (int rc = launch_class<MODE, BF, 8, 16, COMP>(p, A, s, &first)) return rc;
-  if (int rc = launch_class<MODE, BF, 7, 16, COMP>(p, A, s, &first)) return rc;
-  if (int rc = launch_class<MODE, BF, 6, 16, COMP>(p, A, s, &first)) return rc;
-  if (int rc = launch_class<MODE, BF, 5, 16, COMP>(p, A, s, &first)) return rc;
-  if (int rc = launch_class<MODE, BF, 5, 8, COMP>(p, A, s, &first)) return rc;
-  return launch_class<MODE, BF, 4, 8, COMP>(p, A, s, &first);
+  if (int rc = launch_class<MODE, BF, 9, 16, false, COMP>(p, A, s, &first)) return rc;
+  if (int rc = launch_class<MODE, BF, 8, 16, false, COMP>(p, A, s, &first)) return rc;
+  if (int rc = launch_class<MODE, BF, 7, 16, false, COMP>(p, A, s, &first)) return rc;
+  if (int rc = launch_class<MODE, BF, 6, 16, false, COMP>(p, A, s, &first)) return rc;
+  if (int rc = launch_class<MODE, BF, 5, 16, false, COMP>(p, A, s, &first)) return rc;
+  if (int rc = launch_class<MODE, BF, 5, 8, false, COMP>(p, A, s, &first)) return rc;
+  return launch_class<MODE, BF, 4, 8, false, COMP>(p, A, s, &first);
 }
 
 template <int MODE>

@@ -20,7 +20,7 @@ struct HBuildArgs {
   const Unit* units;
   int64_t n_units;
   const unsigned char* rows;
-  int ntc, Jmax, S, logK;  // tiles per side, stencil side
+  int T, ntc, Jmax, S, logK;  // tile side, tiles per side, stencil side
   float2* H;
   int* status;  // bit 4: a tap pair outside the stencil (skipped)
 };
@@ -37,12 +37,12 @@ __global__ void __launch_bounds__(32 * HB_WARPS) holo_build(HBuildArgs A) {
   const int64_t KK = (int64_t)K * K;
   for (int64_t u = blockIdx.x; u < A.n_units; u += gridDim.x) {
     const Unit U = A.units[u];
-    const int r0 = (U.tile / A.ntc) * GT, c0 = (U.tile % A.ntc) * GT;
+    const int r0 = (U.tile / A.ntc) * A.T, c0 = (U.tile % A.ntc) * A.T;
     const int J = U.J, nn = J * J, bytes = 16 * row_units(J, BF);
     if (nn > 256) continue;
     for (int q = wp; q < U.nrows; q += HB_WARPS) {
       const unsigned char* row = A.rows + (U.row_unit << 4) + (size_t)q * bytes;
-      const int cell = row_cell(row, J, BF), lr0 = cell >> 3, lc0 = cell & 7;
+      const int cell = row_cell(row, J, BF), lr0 = (cell >> 5) & (A.T - 1), lc0 = cell & (A.T - 1);
       for (int t = lane; t < nn; t += 32) {
         const int i1 = t / J, i0 = t - i1 * J, lr = lr0 + i1, lc = lc0 + i0;
         s_r[wp][t] = (short)lr;
@@ -137,6 +137,7 @@ int holo_build_plan(pnp_plan* p) {
     A.units = p->d_units;
     A.n_units = p->n_units;
     A.rows = static_cast<const unsigned char*>(p->d_rows);
+    A.T = p->tile;
     A.ntc = p->ntc;
     A.Jmax = p->Jmax;
     A.S = S;

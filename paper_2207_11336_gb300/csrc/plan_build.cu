@@ -34,7 +34,7 @@ struct RowGeom {
   int64_t unit;          // offset of the stored row, 16-byte units
   int s0, s1;            // first tap (unwrapped) per axis
   int J;                 // row support J_m
-  int cell;              // first tap's cell in its tile, row << 3 | column
+  int cell;              // first tap's cell in its coarse tile, row << 5 | column
 };
 
 struct BuildArgs {
@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(256) build_rows(BuildArgs A) {
     if (sl < Jm) {
       const double2 v = s_g[wl][ax][sl];
       if (ax) {
-        const int i1 = sl + ((g.cell >> 3) & 1);
+        const int i1 = sl + ((g.cell >> 5) & 1);
         float* o = out + 4 * (i1 >> 1) + (i1 & 1);
         o[0] = (float)(g.d * v.x);
         o[2] = (float)(g.d * v.y);
@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(256) build_rows(BuildArgs A) {
     const int i1 = t / Jm, i0 = t - i1 * Jm;
     const double2 a = s_g[wl][0][i0], b = s_g[wl][1][i1];
     const float wr = (float)(g.d * (a.x * b.x - a.y * b.y)), wi = (float)(g.d * (a.x * b.y + a.y * b.x));
-    const int e1 = i1 + ((g.cell >> 3) & 1);
+    const int e1 = i1 + ((g.cell >> 5) & 1);
     __nv_bfloat16* o = ob + ((e1 >> 1) * 2 * jp + i0) * 4 + (e1 & 1);
     o[0] = __float2bfloat16_rn(wr);
     o[2] = __float2bfloat16_rn(wi);
@@ -196,6 +196,31 @@ int dev_alloc(pnp_plan* p, T** ptr, size_t count) {
   return PNP_OK;
 }
 
+// Tile side and kind of the work units, from the rows sorted for GT x GT tiles.  Where the units of the classes are thin
+// (few rows of one support in a GT x GT tile), staging and flushing their regions costs more than their rows; larger
+// tiles whose regions all supports share then do better: the cells that the flushes add, a row, fall about threefold.
+// Fused pass, classes -> mixed: 4096^2 grid, uniform coverage, J 7-16: 3e5 rows (1.2 a unit, 5.7 units a 16 x 16 tile)
+// 455 -> 342 us, 1e6 rows (1.9, 12) 899 -> 604 us, 4e6 rows (6.0, 16) 1583 -> 1655 us; a track of 1e5 rows (2.1, 3.9) 108 ->
+// 135 us; 1024^2 grid, 3e4 rows in 2700 tiles (1.4, 7.9) 47 -> 51 us: fewer than two tiles per resident warp (12 an SM).
+void pick_tile(pnp_plan* p) {
+  int64_t units = 0, tiles = 0;
+  int32_t key = -1;
+  int run = -1, seen = 0;  // (sub-tile, support) of the unit; 16 x 16 tiles of the key's coarse tile met so far
+  for (int64_t r = 0; r < p->M; ++r) {
+    const int sub = p->h_start[r] >> 6, u = sub << 8 | p->h_J[r];
+    if (p->h_key[r] == key && u == run) continue;
+    if (p->h_key[r] != key) seen = 0;
+    key = p->h_key[r];
+    run = u;
+    ++units;
+    const int bit = 1 << ((sub / (GKT / GT) * GT / MIX_TILE) * (GKT / MIX_TILE) + sub % (GKT / GT) * GT / MIX_TILE);
+    tiles += (seen & bit) == 0;
+    seen |= bit;
+  }
+  p->mixed = p->M < 3 * units && units >= 5 * tiles && tiles >= (int64_t)24 * p->num_sms * p->nstacks;
+  p->tile = p->mixed ? MIX_TILE : GT;
+}
+
 }  // namespace
 
 int build_units(pnp_plan* p) {
@@ -207,28 +232,42 @@ int build_units(pnp_plan* p) {
   // less where the class is small, so that every resident warp (16 to 24 per SM) gets several units, but
   // enough rows to pay for staging and flushing the unit's region.
   int64_t cap[TAP_CLASSES] = {};
-  for (int64_t r = 0; r < M; ++r) cap[tap_class(tap_pairs(p->h_J[r]), tap_lanes(p->h_J[r]))] += p->h_J[r] * p->h_J[r];
+  for (int64_t r = 0; r < M; ++r)
+    cap[p->mixed ? 0 : tap_class(tap_pairs(p->h_J[r]), tap_lanes(p->h_J[r]))] += p->h_J[r] * p->h_J[r];
   for (int64_t& c : cap)
     c = std::min<int64_t>(p->unit_nnz, std::max<int64_t>(2048, std::min<int64_t>(p->unit_nnz / 8, c / (p->num_sms * 100))));
-  const int cpt = p->K / GKT, per = GKT / GT;  // coarse tiles per side, tiles per coarse tile side
+  const int T = p->tile, cpt = p->K / GKT, per = GKT / T;  // coarse tiles per side, tiles per coarse tile side
+  // tile of a row within its coarse tile: row * per + column
+  auto tile_of = [&](int64_t r) {
+    const int sub = p->h_start[r] >> 6, s1 = sub / (GKT / GT), s0 = sub % (GKT / GT);
+    return s1 * GT / T * per + s0 * GT / T;
+  };
   int64_t i = 0;
   for (int st = 0; st < p->nstacks; ++st) {
+    int32_t last_key = -1;
+    int last_t = -1;
+    int64_t held = 0;  // mixed: taps of the tile's units since the last `first`
     while (i < M && p->h_key[i] / p->nkeys == st) {
       const int32_t key = p->h_key[i];
-      const int sub = p->h_start[i] >> 6, J = p->h_J[i], ct = (int)((key % p->nkeys) / p->nblocks);
+      const int t = tile_of(i), J = p->h_J[i], ct = (int)((key % p->nkeys) / p->nblocks);
       Unit u{};
       u.row_begin = i;
       u.row_unit = p->h_unit[i];
       u.J = J;
-      u.tile = ((ct / cpt) * per + sub / per) * p->ntc + (ct % cpt) * per + sub % per;
-      const int c = tap_class(tap_pairs(J), tap_lanes(J));
+      u.tile = ((ct / cpt) * per + t / per) * p->ntc + (ct % cpt) * per + t % per;
+      const int c = p->mixed ? 0 : tap_class(tap_pairs(J), tap_lanes(J));
       int64_t taps = 0;
-      while (i < M && p->h_key[i] == key && (p->h_start[i] >> 6) == sub && p->h_J[i] == J &&
+      while (i < M && p->h_key[i] == key && tile_of(i) == t && p->h_J[i] == J &&
              (taps == 0 || taps + (int64_t)J * J <= cap[c])) {
         taps += (int64_t)J * J;
         ++u.nrows;
         ++i;
       }
+      held += taps;
+      u.first = !p->mixed || key != last_key || t != last_t || held > cap[c];
+      if (u.first) held = taps;
+      last_key = key;
+      last_t = t;
       cls[c].push_back(u);
     }
     for (auto& v : cls) {
@@ -270,8 +309,7 @@ int plan_build(pnp_plan* p, const double* uvw, const int8_t* Jrow, const int32_t
   }
 
   // per-row geometry, keys
-  const int ntc = K / GT, cpt = K / GKT;  // tiles and coarse tiles per grid side
-  p->ntc = ntc;
+  const int cpt = K / GKT;  // coarse tiles per grid side
   std::vector<RowGeom> geom(M);
   std::vector<int32_t> key(M);
   std::vector<uint16_t> startc(M);  // tile within the coarse tile << 6 | first tap's cell within the tile
@@ -309,61 +347,74 @@ int plan_build(pnp_plan* p, const double* uvw, const int8_t* Jrow, const int32_t
     geom[m] = g;
   }
   p->Jmax = Jmax;
-  p->pitch = GT - tap_quant(tap_pairs(Jmax), tap_lanes(Jmax)) + tap_lanes(Jmax);
 
-  // stable LSD counting sort: by (tile within the coarse tile, support J, first tap's cell in the tile with
-  // the cells of one gridding window together), then by (coarse tile, block) key, so that the rows of one
-  // tile come out grouped by J and, within that, rows sharing a window are adjacent (the gridding pass
-  // keeps it in registers)
-  std::vector<int32_t> by_j(M);
-  {
-    auto bin = [&](int64_t m) {
-      const int J = geom[m].J, q = tap_quant(tap_pairs(J), tap_lanes(J)), c = startc[m] & 63, lr = c >> 3, lc = c & 7;
-      return ((startc[m] >> 6) * 17 + J) * 64 + (((lr >> 1) * (GT / q) + lc / q) * 2 + (lr & 1)) * q + lc % q;
-    };
-    std::vector<int64_t> cc((GKT / GT) * (GKT / GT) * 17 * 64 + 1, 0);
-    for (int64_t m = 0; m < M; ++m) cc[bin(m) + 1]++;
-    for (size_t c = 1; c < cc.size(); ++c) cc[c] += cc[c - 1];
-    for (int64_t m = 0; m < M; ++m) by_j[cc[bin(m)]++] = (int32_t)m;
-  }
   const int64_t nkeys = (int64_t)cpt * cpt * p->nblocks;
   if (nkeys * p->nstacks > INT32_MAX) return fail(PNP_ERR_UNSUPPORTED, "too many (stack, tile, block) keys");
   p->nkeys = nkeys;
-  std::vector<int64_t> cnt(nkeys + 1, 0);
-  for (int64_t m = 0; m < M; ++m) cnt[key[m] + 1]++;
-  for (int64_t k = 0; k < nkeys; ++k) cnt[k + 1] += cnt[k];
-  p->h_perm.assign(M, 0);
-  p->h_inv.assign(M, 0);
-  for (int64_t i = 0; i < M; ++i) {
-    const int32_t m = by_j[i];
-    p->h_perm[cnt[key[m]]++] = m;
-  }
-  if (stack && p->nstacks > 1) {  // most significant: the w-stack
-    std::vector<int64_t> cs(p->nstacks + 1, 0);
-    for (int64_t m = 0; m < M; ++m) cs[stack[m] + 1]++;
-    for (int s = 0; s < p->nstacks; ++s) cs[s + 1] += cs[s];
-    for (int64_t i = 0; i < M; ++i) {
-      const int32_t m = p->h_perm[i];
-      by_j[cs[stack[m]]++] = m;
+  // stable LSD counting sort: by (T x T tile within the coarse tile, support J, first tap's cell in the tile with the
+  // cells of one gridding window together), then by (coarse tile, block) key and w-stack, so that the rows of one
+  // tile come out grouped by J and, within that, rows sharing a window are adjacent (the gridding pass
+  // keeps it in registers)
+  auto sort_rows = [&](int T) {
+    const int per = GKT / T;
+    std::vector<int32_t> by_j(M);
+    {
+      auto bin = [&](int64_t m) {
+        const int J = geom[m].J, q = T == GT ? tap_quant(tap_pairs(J), tap_lanes(J)) : 1;
+        const int sub = startc[m] >> 6, cell = startc[m] & 63;
+        const int r = sub / (GKT / GT) * GT + (cell >> 3), c = sub % (GKT / GT) * GT + (cell & 7);  // in the coarse tile
+        const int lr = r % T, lc = c % T;
+        return ((r / T * per + c / T) * 17 + J) * T * T + (((lr >> 1) * (T / q) + lc / q) * 2 + (lr & 1)) * q + lc % q;
+      };
+      std::vector<int64_t> cc((size_t)17 * GKT * GKT + 1, 0);
+      for (int64_t m = 0; m < M; ++m) cc[bin(m) + 1]++;
+      for (size_t c = 1; c < cc.size(); ++c) cc[c] += cc[c - 1];
+      for (int64_t m = 0; m < M; ++m) by_j[cc[bin(m)]++] = (int32_t)m;
     }
-    p->h_perm.swap(by_j);
-  }
+    std::vector<int64_t> cnt(nkeys + 1, 0);
+    for (int64_t m = 0; m < M; ++m) cnt[key[m] + 1]++;
+    for (int64_t k = 0; k < nkeys; ++k) cnt[k + 1] += cnt[k];
+    p->h_perm.assign(M, 0);
+    for (int64_t i = 0; i < M; ++i) {
+      const int32_t m = by_j[i];
+      p->h_perm[cnt[key[m]]++] = m;
+    }
+    if (stack && p->nstacks > 1) {  // most significant: the w-stack
+      std::vector<int64_t> cs(p->nstacks + 1, 0);
+      for (int64_t m = 0; m < M; ++m) cs[stack[m] + 1]++;
+      for (int s = 0; s < p->nstacks; ++s) cs[s + 1] += cs[s];
+      for (int64_t i = 0; i < M; ++i) {
+        const int32_t m = p->h_perm[i];
+        by_j[cs[stack[m]]++] = m;
+      }
+      p->h_perm.swap(by_j);
+    }
+    p->h_key.assign(M, 0);
+    p->h_start.assign(M, 0);
+    p->h_J.assign(M, 0);
+    for (int64_t i = 0; i < M; ++i) {
+      const int64_t m = p->h_perm[i];
+      p->h_key[i] = (int32_t)((stack ? (int64_t)stack[m] : 0) * nkeys + key[m]);
+      p->h_start[i] = startc[m];
+      p->h_J[i] = (uint8_t)geom[m].J;
+    }
+  };
+  sort_rows(GT);
+  pick_tile(p);
+  if (p->tile != GT) sort_rows(p->tile);
+  p->ntc = K / p->tile;
+  p->pitch = p->mixed ? p->tile - 1 + 16 : GT - tap_quant(tap_pairs(Jmax), tap_lanes(Jmax)) + tap_lanes(Jmax);
+  p->h_inv.assign(M, 0);
   for (int64_t i = 0; i < M; ++i) p->h_inv[p->h_perm[i]] = (int32_t)i;
-  std::vector<int32_t>().swap(by_j);
   std::vector<RowGeom> sgeom(M);
-  p->h_key.assign(M, 0);
-  p->h_start.assign(M, 0);
   p->h_unit.assign(M + 1, 0);
-  p->h_J.assign(M, 0);
   p->nnz = 0;
   for (int64_t i = 0; i < M; ++i) {
     const int64_t m = p->h_perm[i];
     sgeom[i] = geom[m];
-    p->h_key[i] = (int32_t)((stack ? (int64_t)stack[m] : 0) * nkeys + key[m]);
-    p->h_start[i] = startc[m];
-    p->h_J[i] = (uint8_t)geom[m].J;
     sgeom[i].unit = p->h_unit[i];
-    sgeom[i].cell = startc[m] & 63;
+    const int sub = startc[m] >> 6, cell = startc[m] & 63;
+    sgeom[i].cell = (sub / (GKT / GT) * GT + (cell >> 3)) << 5 | (sub % (GKT / GT) * GT + (cell & 7));
     p->h_unit[i + 1] = p->h_unit[i] + row_units(geom[m].J, p->wdtype == PNP_W_BF16C);
     p->nnz += (int64_t)geom[m].J * geom[m].J;
   }

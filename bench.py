@@ -854,11 +854,10 @@ def cnn_case(args):
 
     ms = timed()
     by_rows = {}
-    for rows in (16, 24, 32, 48, 64, 96):   # the strip heights the autotuner chooses among
+    for rows in (16, 24, 32, 48, 64, 96, 1024):   # the strip heights the autotuner chooses among
         den.set_strip_rows(rows)
         den.denoise(z, out)
         by_rows[rows] = timed()
-    den.set_strip_rows(32)
     px = _facet_pixels(n, prob["facet_rows"], prob["facet_cols"], 32)
     flop = px * CNN_FLOP_PER_PX
     print(json.dumps({"case": f"cnn {n}^2, 16 facets, halo 32", "ms": ms, "pixels_with_halo": int(px),

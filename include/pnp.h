@@ -329,8 +329,10 @@ int pnp_den_create_cnn(pnp_den** den, const float* weights_host,
  * Synchronises the device (work lists in use by launches in flight are not overwritten). */
 int pnp_den_cnn_set_strip_rows(pnp_den* den, int rows);
 /* Autotuner of the strip height above: times `reps` denoises (after one warm-up) of the device
- * n x n image z for each of 16, 24, 32, 48, 64 and 96 rows on the denoiser's stream (CUDA events),
- * keeps the fastest and returns it with its time per denoise (rows_out, ms_out may be NULL).
+ * n x n image z on the denoiser's stream (CUDA events) for the present height, 16, 24, 32, 48, 64, 96
+ * and 1024 rows, keeps the present work lists unless others are faster, and returns the height with
+ * its time per denoise (rows_out, ms_out may be NULL).  Heights that give the same work lists are timed
+ * once and returned as the smallest of them.
  * Allocates and frees one n x n scratch image.  reps in [1, 100]. */
 int pnp_den_cnn_autotune(pnp_den* den, const float* z, int n, int reps, int* rows_out, double* ms_out);
 

@@ -574,7 +574,7 @@ class CnnDenoiser(_Denoiser):
         _check(lib().pnp_den_cnn_set_strip_rows(self._h, int(rows)))
 
     def autotune(self, z, reps: int = 3) -> dict:
-        """Time the denoise of the device image z for each strip height and keep the fastest."""
+        """Time the denoise of the device image z at the present strip height and the others and keep the fastest."""
         _cuda_f32(z, (self.n, self.n), "z")
         rows, ms = C.c_int(), C.c_double()
         _check(lib().pnp_den_cnn_autotune(self._h, _ptr(z), self.n, int(reps), C.byref(rows), C.byref(ms)))

@@ -516,7 +516,7 @@ __global__ void __launch_bounds__(256) cnn_first(FirstArgs A) {
 // a 3 x 3 gather N[y][x] = b8 + sum_t P[y + dy - 1][x + dx - 1][t] (t = 3 dy + dx) from a ring of
 // three projected rows in shared memory, fused with D(z) = max(0, z - N(z)) and the FP64
 // stopping-test sums.  A CTA walks one strip of the last layer's work list (128 core columns x
-// about 32 core rows of a facet) row by row; P covers the 144 pixels x0 - 1 .. x0 + 142 of each
+// up to 128 core rows of a facet) row by row; P covers the 144 pixels x0 - 1 .. x0 + 142 of each
 // activation row (9 M tiles of 16), so the gather never leaves the CTA.  Each activation row is
 // copied into shared memory with cp.async (16-byte pieces, whole runs of each channel block's
 // plane, zero-filled outside the facet) one row ahead of its projection, double buffered, and the
@@ -735,14 +735,18 @@ int sms_of_device() {
 
 }  // namespace
 
-// The two convolution work lists for strips of about `rows` output rows: the hidden layers' strips of
-// the extended facets, and the last layer's strips of the facet cores.  Device arrays grow as needed.
-static int build_strips(CnnState* S, int rows) {
+// The two convolution work lists for strips of at most `rows` output rows: the hidden layers' strips of
+// the extended facets, and the last layer's strips of the facet cores.
+struct StripLists {
+  std::vector<int4> hidden, last;
+  int grid = 0;  // CTAs of the hidden layers
+};
+static StripLists strip_lists(const CnnState* S, int rows) {
   const int sms = sms_of_device();
-  const std::vector<int4> strips = conv_strips(S->F, S->Hf.data(), S->Wf.data(), sms, &S->conv_grid, rows);
+  StripLists out;
+  out.hidden = conv_strips(S->F, S->Hf.data(), S->Wf.data(), sms, &out.grid, rows);
   // last layer: strips of the cores of at most `rows` rows, of the height (8 .. 128) at which the resident CTAs
   // (four per SM) share the staged rows best: rounds x (rows + 2 halo rows)
-  std::vector<int4> lstrips;
   int best = 0;
   int64_t best_cost = -1;
   for (int h = 8; h <= 128; ++h) {
@@ -766,9 +770,16 @@ static int build_strips(CnnState* S, int rows) {
     for (int x0 = cc0; x0 < cc1; x0 += TILE_PX)
       for (int i = 0; i < k; ++i) {
         const int ya = cr0 + (int)((int64_t)(cr1 - cr0) * i / k), yb = cr0 + (int)((int64_t)(cr1 - cr0) * (i + 1) / k);
-        if (yb > ya) lstrips.push_back(make_int4(f, x0, (ya << 16) | (yb - ya), (S->Hf[f] << 16) | S->Wf[f]));
+        if (yb > ya) out.last.push_back(make_int4(f, x0, (ya << 16) | (yb - ya), (S->Hf[f] << 16) | S->Wf[f]));
       }
   }
+  return out;
+}
+
+// Installs the work lists for strips of at most `rows` rows.  Device arrays grow as needed.
+static int build_strips(CnnState* S, int rows) {
+  const StripLists lists = strip_lists(S, rows);
+  const std::vector<int4>&strips = lists.hidden, &lstrips = lists.last;
   auto fit = [](void** p, size_t* cap, size_t need, size_t item) -> int {
     need = std::max<size_t>(1, need);
     if (*p && *cap >= need) return PNP_OK;
@@ -789,6 +800,7 @@ static int build_strips(CnnState* S, int rows) {
     PNP_CUDA(cudaMemcpy(S->d_strips, strips.data(), strips.size() * sizeof(int4), cudaMemcpyHostToDevice));
   if (!lstrips.empty())
     PNP_CUDA(cudaMemcpy(S->d_lstrips, lstrips.data(), lstrips.size() * sizeof(int4), cudaMemcpyHostToDevice));
+  S->conv_grid = lists.grid;
   S->n_strips = (int)strips.size();
   S->n_lstrips = (int)lstrips.size();
   S->strip_rows = rows;
@@ -995,7 +1007,7 @@ int conv64_launch(cudaStream_t s, const void* in_map, __nv_bfloat16* out, const 
 std::vector<int4> conv_strips(int F, const int* Hf, const int* Wf, int sms, int* grid_out, int rows) {
   int64_t total = 0;
   for (int f = 0; f < F; ++f) total += (int64_t)((Wf[f] + TILE_PX - 1) / TILE_PX) * Hf[f];
-  // at least four rows per CTA: below that the halo rows outweigh what another SM adds
+  // at least four rows per CTA: below that the halo rows outweigh what another SM adds (lower `rows` cut further)
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(sms, total / 4));
   const int64_t shares = grid * std::max<int64_t>(1, (total + (int64_t)grid * rows - 1) / ((int64_t)grid * rows));
   std::vector<std::vector<int4>> cta(grid);
@@ -1018,7 +1030,8 @@ std::vector<int4> conv_strips(int F, const int* Hf, const int* Wf, int sms, int*
       size_t t = 0;
       for (size_t k = 1; k < c.size(); ++k)
         if ((c[k].z & 0xFFFF) > (c[t].z & 0xFFFF)) t = k;
-      const int y = c[t].z >> 16, n = c[t].z & 0xFFFF, h = n / 2;  // n >= 2: a share has four rows or more
+      // a strip of one row (facets of a row or two, low heights) leaves an empty one: it stages two rows and stores none
+      const int y = c[t].z >> 16, n = c[t].z & 0xFFFF, h = n / 2;
       int4 lower = c[t];
       lower.z = ((y + h) << 16) | (n - h);
       c[t].z = (y << 16) | h;
@@ -1053,6 +1066,32 @@ int cnn_set_strip_rows(pnp_den* d, int rows) {
 int cnn_strip_rows(pnp_den* d) {
   const CnnState* S = static_cast<const CnnState*>(d->impl);
   return S ? S->strip_rows : 0;
+}
+
+std::vector<int> cnn_strip_candidates(pnp_den* d) {
+  const CnnState* S = static_cast<const CnnState*>(d->impl);
+  std::vector<int> heights{16, 24, 32, 48, 64, 96, STRIP_ROWS};
+  if (!S) return heights;
+  heights.push_back(S->strip_rows);
+  std::sort(heights.begin(), heights.end());
+  auto same = [](const std::vector<int4>& a, const std::vector<int4>& b) {
+    return a.size() == b.size() && (a.empty() || !memcmp(a.data(), b.data(), a.size() * sizeof(int4)));
+  };
+  std::vector<StripLists> seen;
+  std::vector<int> out;
+  size_t now = 0;  // the present lists' entry
+  for (int h : heights) {
+    StripLists l = strip_lists(S, h);
+    size_t k = 0;
+    while (k < seen.size() && !(same(seen[k].hidden, l.hidden) && same(seen[k].last, l.last))) ++k;
+    if (k == seen.size()) {
+      seen.push_back(std::move(l));
+      out.push_back(h);
+    }
+    if (h == S->strip_rows) now = k;
+  }
+  std::rotate(out.begin(), out.begin() + now, out.begin() + now + 1);
+  return out;
 }
 
 int cnn_status(pnp_den* d, int* flags) {

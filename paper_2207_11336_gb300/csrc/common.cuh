@@ -253,6 +253,8 @@ std::vector<int4> conv_strips(int F, const int* Hf, const int* Wf, int sms, int*
 // the denoiser's convolution work lists rebuilt for strips of at most `rows` output rows (4..1024)
 int cnn_set_strip_rows(pnp_den* d, int rows);
 int cnn_strip_rows(pnp_den* d);
+// strip heights with different work lists: the present ones' first, each the smallest of those with the same lists
+std::vector<int> cnn_strip_candidates(pnp_den* d);
 // the convolution reads its input through the TMA descriptor in_map (canvas_map_create)
 int conv64_launch(cudaStream_t s, const void* in_map, __nv_bfloat16* out, const __nv_bfloat16* w_packed,
                   const float* bias, const int4* strips, int n_strips, int grid, int Hc, int Wc, int mode,

@@ -583,20 +583,20 @@ int pnp_den_cnn_set_strip_rows(pnp_den* den, int rows) {
 int pnp_den_cnn_autotune(pnp_den* den, const float* z, int n, int reps, int* rows_out, double* ms_out) {
   if (!den || den->kind != PNP_DEN_CNN || !z) return fail(PNP_ERR_INVALID_ARG, "not a CNN denoiser, or NULL input");
   if (reps < 1 || reps > 100) return fail(PNP_ERR_INVALID_ARG, "reps must lie in [1, 100]");
-  static const int kRows[] = {16, 24, 32, 48, 64, 96};
   float* out = nullptr;
   if (cudaMalloc(&out, (size_t)n * n * sizeof(float)) != cudaSuccess) {
     cudaGetLastError();
     return fail(PNP_ERR_OOM, "autotune scratch image");
   }
   cudaEvent_t e0 = nullptr, e1 = nullptr;
-  int rc = PNP_OK, best = cnn_strip_rows(den);
+  const int old = cnn_strip_rows(den);
+  int rc = PNP_OK, best = old;
   double best_ms = -1.0;
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
     cudaGetLastError();
     rc = fail(PNP_ERR_CUDA, "event creation failed");
   }
-  for (int rows : kRows) {
+  for (int rows : cnn_strip_candidates(den)) {  // the present lists first: kept unless others are faster
     if (rc) break;
     if ((rc = cnn_set_strip_rows(den, rows))) break;
     if ((rc = cnn_denoise(den, den->stream, z, out, n, nullptr, nullptr))) break;  // warm
@@ -618,7 +618,7 @@ int pnp_den_cnn_autotune(pnp_den* den, const float* z, int n, int reps, int* row
   if (e0) cudaEventDestroy(e0);
   if (e1) cudaEventDestroy(e1);
   cudaFree(out);
-  if (!rc) rc = cnn_set_strip_rows(den, best);
+  if (const int rc2 = cnn_set_strip_rows(den, rc ? old : best)) rc = rc ? rc : rc2;
   den->serial = ++g_den_serial;
   if (rc) return rc;
   if (rows_out) *rows_out = best;

@@ -381,7 +381,6 @@ int pnp_plan_set_row_batch(pnp_plan* p, int row_batch) {
     return fail(PNP_ERR_INVALID_ARG, "row_batch must be 0, 1, 2 or 4");
   if (row_batch == 0) return PNP_OK;
   PNP_CUDA(cudaStreamSynchronize(p->stream));
-  if (row_batch != p->row_batch) ++p->epoch;
   p->row_batch = row_batch;
   return PNP_OK;
 }

@@ -269,7 +269,9 @@ int pnp_plan_device_status(pnp_plan* plan, int* flags_host);
 int pnp_plan_set_timing(pnp_plan* plan, int enable);
 int pnp_plan_read_timing(pnp_plan* plan, double* ms_host /*[3]*/, int64_t* count_host /*[3]*/);
 
-/* Copy rows of G to the host for inspection (synchronous).
+/* Copy rows of G to the host for inspection (synchronous): the definition's
+ * weights rounded once to complex64, and from there to bfloat16 in such plans.
+ * (The gridding pass of a complex64 plan multiplies two rounded factors per tap.)
  *  rows_host      host, nrows row indices in the caller's order
  *  offsets_host   host, nrows+1 int64: written with exclusive prefix sums of J_m^2
  *  weights_host   host, offsets_host[nrows] complex64 (interleaved)

@@ -97,6 +97,10 @@ __device__ __forceinline__ float2 row_tap(const unsigned char* row, int J, bool 
   return cmul(make_float2(f[4 * jp + 2 * i0], f[4 * jp + 2 * i0 + 1]), make_float2(g1[0], g1[2]));
 }
 
+// What the taps of a row follow from: kappa per axis, chirp rate a = w dl^2, data weight
+struct RowKey {
+  double kap0, kap1, a, d;
+};
 struct Unit {
   long long row_begin;  // first row (sorted order)
   long long row_unit;   // its offset in the stored rows, 16-byte units
@@ -157,6 +161,9 @@ struct pnp_plan {
                                          // they are ~2^-24 of the sums); kept zero between uses
   bool compensated = false;    // gridding flushes add their rounding errors to d_gridB_lo (TwoSum)
   float2* d_tmp = nullptr;     // K*n: half-transformed intermediate
+  double* d_mu = nullptr;      // the w-kernel series: moments [nterms][2 D + 1], scale, centre
+  int nterms = 0, series_D = 0;
+  double bscale = 0, series_c0 = 0;
   void* d_rows = nullptr;      // stored rows of G in sorted order (row_units 16-byte units each)
   unsigned* d_sched = nullptr; // unit counters of the gridding kernels, two per stack and class (zero at rest)
   int32_t* d_perm = nullptr;   // sorted row -> caller row
@@ -164,7 +171,7 @@ struct pnp_plan {
   pnp::Unit* d_units = nullptr;
   int64_t n_units = 0;
   double* d_acc = nullptr;     // FP64 accumulators [8]
-  int* d_status = nullptr;     // device status flags [4] (bit 0: gridding index out of range)
+  int* d_status = nullptr;     // device status flags [4] (pnp_plan_device_status)
   float* d_img[3] = {nullptr, nullptr, nullptr};  // n*n work images
   float2* d_chirp = nullptr;   // P*n (P > 1): per stack and image axis exp(i pi a_p (a - n/2)^2)
   float* d_gacc = nullptr;     // n*n (P > 1): gradient image accumulated over the stacks
@@ -190,6 +197,7 @@ struct pnp_plan {
   // host mirrors used by export and work-list rebuilds
   std::vector<int64_t> h_unit;     // M+1: offsets of the stored rows, 16-byte units
   std::vector<uint8_t> h_J;        // sorted: support of the row
+  std::vector<pnp::RowKey> h_rowkey;  // caller order, for export
   std::vector<int32_t> h_perm;     // sorted -> caller
   std::vector<int32_t> h_inv;      // caller -> sorted
   std::vector<int32_t> h_key;      // sorted: (stack * coarse tiles + coarse tile) * nblocks + block

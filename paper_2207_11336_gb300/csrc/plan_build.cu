@@ -28,10 +28,8 @@ namespace {
 constexpr int MAX_TERMS = 64;
 constexpr int MAX_D = 15;  // |d| <= MAX_D, so 2 MAX_D + 1 <= 32 lanes
 
-struct RowGeom {
-  double kap0, kap1, a;  // kappa per axis, chirp rate a = w dl^2
-  double d;              // data weight d_m multiplying the row (1 without weighting)
-  int64_t unit;          // offset of the stored row, 16-byte units
+struct RowGeom : RowKey {
+  int64_t unit;          // offset of the stored row, 16-byte units (export: of the row's taps)
   int s0, s1;            // first tap (unwrapped) per axis
   int J;                 // row support J_m
   int cell;              // first tap's cell in its coarse tile, row << 5 | column
@@ -46,6 +44,9 @@ struct BuildArgs {
   const RowGeom* geom;       // sorted order
   unsigned char* rows;       // stored rows (zero: the padding stays)
   int bf16;
+  float2* taps;              // export: the J x J taps (k1-major) in the place of the stored rows, and their columns
+  int32_t* cols;
+  int logK;
 };
 
 __device__ __forceinline__ double kb_psi(double t, int J, double beta) {
@@ -107,6 +108,18 @@ __global__ void __launch_bounds__(256) build_rows(BuildArgs A) {
     s_g[wl][ax][sl] = make_double2(gr, gi);
   }
   __syncwarp();
+  if (A.taps) {
+    const int Km = (1 << A.logK) - 1;
+    for (int t = lane; t < Jm * Jm; t += 32) {
+      const int i1 = t / Jm, i0 = t - i1 * Jm;
+      const double2 a = s_g[wl][0][i0], b = s_g[wl][1][i1];
+      float2 w = make_float2((float)(g.d * (a.x * b.x - a.y * b.y)), (float)(g.d * (a.x * b.y + a.y * b.x)));
+      if (A.bf16) w = __bfloat1622float2(__floats2bfloat162_rn(w.x, w.y));
+      A.taps[g.unit + t] = w;
+      A.cols[g.unit + t] = (((g.s0 + i0) & Km) << A.logK) | ((g.s1 + i1) & Km);
+    }
+    return;
+  }
   const int jp = tap_pairs(Jm);
   float* out = reinterpret_cast<float*>(A.rows + (g.unit << 4));
   if (!A.bf16) {
@@ -136,24 +149,6 @@ __global__ void __launch_bounds__(256) build_rows(BuildArgs A) {
     __nv_bfloat16* o = ob + ((e1 >> 1) * 2 * jp + i0) * 4 + (e1 & 1);
     o[0] = __float2bfloat16_rn(wr);
     o[2] = __float2bfloat16_rn(wi);
-  }
-}
-
-// gather rows for export: canonical column order k0*K + k1, float weights.  src_off holds per
-// row (offset of the stored row, support, first tap's k1, first tap's k0).
-__global__ void export_rows(const int64_t* __restrict__ src_off, const int64_t* __restrict__ dst_off,
-                            int64_t nrows, const unsigned char* rows, int bf16, int logK, float2* out_w,
-                            int32_t* out_c) {
-  const int64_t r = blockIdx.x;
-  if (r >= nrows) return;
-  const unsigned char* row = rows + (src_off[4 * r] << 4);
-  const int64_t d = dst_off[r];
-  const int J = (int)src_off[4 * r + 1], r0 = (int)src_off[4 * r + 2], c0 = (int)src_off[4 * r + 3];
-  const int Km = (1 << logK) - 1;
-  for (int t = threadIdx.x; t < J * J; t += blockDim.x) {
-    const int i1 = t / J, i0 = t - i1 * J;
-    out_w[d + t] = row_tap(row, J, bf16 != 0, i1, i0);
-    out_c[d + t] = (((c0 + i0) & Km) << logK) | ((r0 + i1) & Km);
   }
 }
 
@@ -195,6 +190,25 @@ int dev_alloc(pnp_plan* p, T** ptr, size_t count) {
   p->device_bytes += (int64_t)(count * sizeof(T));
   return PNP_OK;
 }
+
+BuildArgs build_args(const pnp_plan* p, int64_t nrows, const RowGeom* d_geom) {
+  BuildArgs A{};
+  A.M = nrows;
+  A.J = p->J;
+  A.beta = p->beta;
+  A.bscale = p->bscale;
+  A.c0 = p->series_c0;
+  A.nterms = p->nterms;
+  A.D = p->series_D;
+  A.mu = p->d_mu;
+  A.geom = d_geom;
+  A.bf16 = p->wdtype == PNP_W_BF16C;
+  A.logK = p->logK;
+  return A;
+}
+
+// first tap per axis of a row of support J
+int first_tap(double kap, int J) { return (int)std::floor(kap - 0.5 * J) + 1; }
 
 // Tile side and kind of the work units, from the rows sorted for GT x GT tiles.  Where the units of the classes are thin
 // (few rows of one support in a GT x GT tile), staging and flushing their regions costs more than their rows; larger
@@ -311,6 +325,7 @@ int plan_build(pnp_plan* p, const double* uvw, const int8_t* Jrow, const int32_t
   // per-row geometry, keys
   const int cpt = K / GKT;  // coarse tiles per grid side
   std::vector<RowGeom> geom(M);
+  p->h_rowkey.resize(M);
   std::vector<int32_t> key(M);
   std::vector<uint16_t> startc(M);  // tile within the coarse tile << 6 | first tap's cell within the tile
   int Jmax = J;
@@ -336,8 +351,8 @@ int plan_build(pnp_plan* p, const double* uvw, const int8_t* Jrow, const int32_t
       return fail(PNP_ERR_INVALID_ARG, "J_per_row must lie in [J, 16]; row " + std::to_string(m));
     if (block && (block[m] < 0 || block[m] >= p->nblocks))
       return fail(PNP_ERR_INVALID_ARG, "block id out of range at row " + std::to_string(m));
-    g.s0 = (int)std::floor(g.kap0 - 0.5 * g.J) + 1;
-    g.s1 = (int)std::floor(g.kap1 - 0.5 * g.J) + 1;
+    g.s0 = first_tap(g.kap0, g.J);
+    g.s1 = first_tap(g.kap1, g.J);
     const int f0 = ((g.s0 % K) + K) % K, f1 = ((g.s1 % K) + K) % K;
     key[m] = ((f1 / GKT) * cpt + (f0 / GKT)) * p->nblocks + (block ? block[m] : 0);
     const int sub = (f1 % GKT) / GT * (GKT / GT) + (f0 % GKT) / GT;
@@ -345,6 +360,7 @@ int plan_build(pnp_plan* p, const double* uvw, const int8_t* Jrow, const int32_t
     Jmax = std::max(Jmax, g.J);
     amax = std::max(amax, std::fabs(g.a));
     geom[m] = g;
+    p->h_rowkey[m] = g;
   }
   p->Jmax = Jmax;
 
@@ -561,33 +577,24 @@ int plan_build(pnp_plan* p, const double* uvw, const int8_t* Jrow, const int32_t
   // build G rows on the GPU
   if (M) {
     RowGeom* d_geom = nullptr;
-    double* d_mu = nullptr;
-    if (cudaMalloc(&d_geom, M * sizeof(RowGeom)) != cudaSuccess ||
-        cudaMalloc(&d_mu, mu.size() * sizeof(double)) != cudaSuccess) {
+    if (int rc = dev_alloc(p, &p->d_mu, mu.size())) return rc;
+    if (cudaMalloc(&d_geom, M * sizeof(RowGeom)) != cudaSuccess) {
       cudaGetLastError();
-      cudaFree(d_geom);
       return fail(PNP_ERR_OOM, "plan build scratch allocation failed");
     }
     PNP_CUDA(cudaMemcpy(d_geom, sgeom.data(), M * sizeof(RowGeom), cudaMemcpyHostToDevice));
-    PNP_CUDA(cudaMemcpy(d_mu, mu.data(), mu.size() * sizeof(double), cudaMemcpyHostToDevice));
-    BuildArgs A{};
-    A.M = M;
-    A.J = J;
-    A.beta = p->beta;
-    A.bscale = bscale;
-    A.c0 = c0;
-    A.nterms = nterms;
-    A.D = D;
-    A.mu = d_mu;
-    A.geom = d_geom;
+    PNP_CUDA(cudaMemcpy(p->d_mu, mu.data(), mu.size() * sizeof(double), cudaMemcpyHostToDevice));
+    p->nterms = nterms;
+    p->series_D = D;
+    p->bscale = bscale;
+    p->series_c0 = c0;
+    BuildArgs A = build_args(p, M, d_geom);
     A.rows = static_cast<unsigned char*>(p->d_rows);
-    A.bf16 = p->wdtype == PNP_W_BF16C;
     build_rows<<<(unsigned)((M + 7) / 8), 256, 0, p->stream>>>(A);
     cudaError_t e = cudaGetLastError();
     g_launches.fetch_add(1);
     if (e == cudaSuccess) e = cudaStreamSynchronize(p->stream);
     cudaFree(d_geom);
-    cudaFree(d_mu);
     if (e != cudaSuccess) return fail(PNP_ERR_CUDA, std::string("build_rows: ") + cudaGetErrorString(e));
   }
   return build_units(p);
@@ -595,49 +602,50 @@ int plan_build(pnp_plan* p, const double* uvw, const int8_t* Jrow, const int32_t
 
 int export_rows_impl(const pnp_plan* p, const int64_t* rows, int64_t nrows, int64_t* offsets,
                      float* weights, int32_t* cols) {
-  std::vector<int64_t> src(4 * nrows), dst(nrows);
+  // evaluated anew in FP64: a stored complex64 row holds two rounded factors, whose products carry 1.8 times the error
+  // (1e4 rows: 0.96 -> 1.55 ms against reading the stored rows)
+  std::vector<RowGeom> geom(weights && cols ? nrows : 0);
   offsets[0] = 0;
   for (int64_t i = 0; i < nrows; ++i) {
     if (rows[i] < 0 || rows[i] >= p->M) return fail(PNP_ERR_INVALID_ARG, "export row index out of range");
-    const int64_t s = p->h_inv[rows[i]];
-    const int ct = (int)((p->h_key[s] % p->nkeys) / p->nblocks), cpt = p->K / GKT, per = GKT / GT;
-    const int sub = p->h_start[s] >> 6, cell = p->h_start[s] & 63;
-    src[4 * i] = p->h_unit[s];
-    src[4 * i + 1] = p->h_J[s];
-    src[4 * i + 2] = (int64_t)(ct / cpt) * GKT + sub / per * GT + (cell >> 3);
-    src[4 * i + 3] = (int64_t)(ct % cpt) * GKT + sub % per * GT + (cell & 7);
-    dst[i] = offsets[i];
-    offsets[i + 1] = offsets[i] + (int64_t)p->h_J[s] * p->h_J[s];
+    RowGeom g{};
+    static_cast<RowKey&>(g) = p->h_rowkey[rows[i]];
+    g.J = p->h_J[p->h_inv[rows[i]]];
+    g.s0 = first_tap(g.kap0, g.J);
+    g.s1 = first_tap(g.kap1, g.J);
+    g.unit = offsets[i];
+    if (!geom.empty()) geom[i] = g;
+    offsets[i + 1] = offsets[i] + (int64_t)g.J * g.J;
   }
   if (!weights || !cols || nrows == 0) return PNP_OK;
   const int64_t total = offsets[nrows];
-  int64_t *d_src = nullptr, *d_dst = nullptr;
+  RowGeom* d_geom = nullptr;
   float2* d_w = nullptr;
   int32_t* d_c = nullptr;
-  if (cudaMalloc(&d_src, 4 * nrows * sizeof(int64_t)) || cudaMalloc(&d_dst, nrows * sizeof(int64_t)) ||
-      cudaMalloc(&d_w, total * sizeof(float2)) || cudaMalloc(&d_c, total * sizeof(int32_t))) {
-    cudaGetLastError();
-    cudaFree(d_src);
-    cudaFree(d_dst);
-    cudaFree(d_w);
-    return fail(PNP_ERR_OOM, "export scratch allocation failed");
-  }
   int rc = PNP_OK;
-  cudaError_t e = cudaMemcpy(d_src, src.data(), 4 * nrows * sizeof(int64_t), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(d_dst, dst.data(), nrows * sizeof(int64_t), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) {
-    export_rows<<<(unsigned)nrows, 128, 0, p->stream>>>(d_src, d_dst, nrows,
-                                                         static_cast<const unsigned char*>(p->d_rows),
-                                                         p->wdtype == PNP_W_BF16C, p->logK, d_w, d_c);
-    g_launches.fetch_add(1);
-    e = cudaGetLastError();
+  if (cudaMalloc(&d_geom, nrows * sizeof(RowGeom)) || cudaMalloc(&d_w, total * sizeof(float2)) ||
+      cudaMalloc(&d_c, total * sizeof(int32_t))) {
+    cudaGetLastError();
+    rc = fail(PNP_ERR_OOM, "export scratch allocation failed");
   }
-  if (e == cudaSuccess) e = cudaStreamSynchronize(p->stream);
-  if (e == cudaSuccess) e = cudaMemcpy(weights, d_w, total * sizeof(float2), cudaMemcpyDeviceToHost);
-  if (e == cudaSuccess) e = cudaMemcpy(cols, d_c, total * sizeof(int32_t), cudaMemcpyDeviceToHost);
-  if (e != cudaSuccess) rc = fail(PNP_ERR_CUDA, std::string("export_rows: ") + cudaGetErrorString(e));
-  cudaFree(d_src);
-  cudaFree(d_dst);
+  if (!rc) {
+    cudaError_t e = cudaMemcpy(d_geom, geom.data(), nrows * sizeof(RowGeom), cudaMemcpyHostToDevice);
+    // a small copy may still be on its way, and p->stream need not wait for it
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
+    if (e == cudaSuccess) {
+      BuildArgs A = build_args(p, nrows, d_geom);
+      A.taps = d_w;
+      A.cols = d_c;
+      build_rows<<<(unsigned)((nrows + 7) / 8), 256, 0, p->stream>>>(A);
+      g_launches.fetch_add(1);
+      e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(p->stream);
+    if (e == cudaSuccess) e = cudaMemcpy(weights, d_w, total * sizeof(float2), cudaMemcpyDeviceToHost);
+    if (e == cudaSuccess) e = cudaMemcpy(cols, d_c, total * sizeof(int32_t), cudaMemcpyDeviceToHost);
+    if (e != cudaSuccess) rc = fail(PNP_ERR_CUDA, std::string("export_rows: ") + cudaGetErrorString(e));
+  }
+  cudaFree(d_geom);
   cudaFree(d_w);
   cudaFree(d_c);
   return rc;

@@ -64,6 +64,7 @@ void free_plan(pnp_plan* p) {
   cudaFree(p->d_gridB_lo);
   cudaFree(p->d_tmp);
   cudaFree(p->d_rows);
+  cudaFree(p->d_mu);
   cudaFree(p->d_sched);
   cudaFree(p->d_perm);
   cudaFree(p->d_ysorted);

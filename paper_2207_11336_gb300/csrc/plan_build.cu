@@ -210,26 +210,31 @@ BuildArgs build_args(const pnp_plan* p, int64_t nrows, const RowGeom* d_geom) {
 // first tap per axis of a row of support J
 int first_tap(double kap, int J) { return (int)std::floor(kap - 0.5 * J) + 1; }
 
-// Tile side and kind of the work units, from the rows sorted for GT x GT tiles.  Where the units of the classes are thin
+// Tile side and kind of the work units, before the rows are sorted for them.  Where the units of the classes are thin
 // (few rows of one support in a GT x GT tile), staging and flushing their regions costs more than their rows; larger
 // tiles whose regions all supports share then do better: the cells that the flushes add, a row, fall about threefold.
 // Fused pass, classes -> mixed: 4096^2 grid, uniform coverage, J 7-16: 3e5 rows (1.2 a unit, 5.7 units a 16 x 16 tile)
 // 455 -> 342 us, 1e6 rows (1.9, 12) 899 -> 604 us, 4e6 rows (6.0, 16) 1583 -> 1655 us; a track of 1e5 rows (2.1, 3.9) 108 ->
 // 135 us; 1024^2 grid, 3e4 rows in 2700 tiles (1.4, 7.9) 47 -> 51 us: fewer than two tiles per resident warp (12 an SM).
-void pick_tile(pnp_plan* p) {
+// key: (coarse tile, block); startc: tile within the coarse tile << 6 | cell; supports: bit J for each J of the plan.
+void pick_tile(pnp_plan* p, const std::vector<RowGeom>& geom, const std::vector<int32_t>& key,
+               const std::vector<uint16_t>& startc, const int32_t* stack, unsigned supports) {
+  constexpr int SUBS = (GKT / GT) * (GKT / GT);
+  const int64_t coarse = p->nkeys * p->nstacks;
+  // too many rows for thin units, or a mask of more than half a gigabyte
+  if (p->M >= 3 * coarse * SUBS * __builtin_popcount(supports) || coarse * SUBS > (int64_t(1) << 28)) return;
+  std::vector<uint16_t> mask(coarse * SUBS, 0);  // per GT x GT tile, block and stack: its supports (bit J - 2)
+  for (int64_t m = 0; m < p->M; ++m)
+    mask[((stack ? (int64_t)stack[m] * p->nkeys : 0) + key[m]) * SUBS + (startc[m] >> 6)] |= (uint16_t)(1u << (geom[m].J - 2));
   int64_t units = 0, tiles = 0;
-  int32_t key = -1;
-  int run = -1, seen = 0;  // (sub-tile, support) of the unit; 16 x 16 tiles of the key's coarse tile met so far
-  for (int64_t r = 0; r < p->M; ++r) {
-    const int sub = p->h_start[r] >> 6, u = sub << 8 | p->h_J[r];
-    if (p->h_key[r] == key && u == run) continue;
-    if (p->h_key[r] != key) seen = 0;
-    key = p->h_key[r];
-    run = u;
-    ++units;
-    const int bit = 1 << ((sub / (GKT / GT) * GT / MIX_TILE) * (GKT / MIX_TILE) + sub % (GKT / GT) * GT / MIX_TILE);
-    tiles += (seen & bit) == 0;
-    seen |= bit;
+  for (int64_t k = 0; k < coarse; ++k) {
+    unsigned seen = 0;  // its MIX_TILE x MIX_TILE tiles with rows
+    for (int sub = 0; sub < SUBS; ++sub) {
+      const unsigned u = mask[k * SUBS + sub];
+      units += __builtin_popcount(u);
+      if (u) seen |= 1u << (sub / (GKT / GT) * GT / MIX_TILE * (GKT / MIX_TILE) + sub % (GKT / GT) * GT / MIX_TILE);
+    }
+    tiles += __builtin_popcount(seen);
   }
   p->mixed = p->M < 3 * units && units >= 5 * tiles && tiles >= (int64_t)24 * p->num_sms * p->nstacks;
   p->tile = p->mixed ? MIX_TILE : GT;
@@ -250,12 +255,11 @@ int build_units(pnp_plan* p) {
     cap[p->mixed ? 0 : tap_class(tap_pairs(p->h_J[r]), tap_lanes(p->h_J[r]))] += p->h_J[r] * p->h_J[r];
   for (int64_t& c : cap)
     c = std::min<int64_t>(p->unit_nnz, std::max<int64_t>(2048, std::min<int64_t>(p->unit_nnz / 8, c / (p->num_sms * 100))));
-  const int T = p->tile, cpt = p->K / GKT, per = GKT / T;  // coarse tiles per side, tiles per coarse tile side
-  // tile of a row within its coarse tile: row * per + column
-  auto tile_of = [&](int64_t r) {
-    const int sub = p->h_start[r] >> 6, s1 = sub / (GKT / GT), s0 = sub % (GKT / GT);
-    return s1 * GT / T * per + s0 * GT / T;
-  };
+  const int cpt = p->K / GKT, per = GKT / p->tile;  // coarse tiles per side, tiles per coarse tile side
+  int of_sub[(GKT / GT) * (GKT / GT)];              // a row's tile within its coarse tile: row * per + column
+  for (int sub = 0; sub < (GKT / GT) * (GKT / GT); ++sub)
+    of_sub[sub] = sub / (GKT / GT) * GT / p->tile * per + sub % (GKT / GT) * GT / p->tile;
+  auto tile_of = [&](int64_t r) { return of_sub[p->h_start[r] >> 6]; };
   int64_t i = 0;
   for (int st = 0; st < p->nstacks; ++st) {
     int32_t last_key = -1;
@@ -325,7 +329,8 @@ int plan_build(pnp_plan* p, const double* uvw, const int8_t* Jrow, const int32_t
   // per-row geometry, keys
   const int cpt = K / GKT;  // coarse tiles per grid side
   std::vector<RowGeom> geom(M);
-  p->h_rowkey.resize(M);
+  p->h_rowkey.reserve(M);
+  unsigned supports = 0;
   std::vector<int32_t> key(M);
   std::vector<uint16_t> startc(M);  // tile within the coarse tile << 6 | first tap's cell within the tile
   int Jmax = J;
@@ -359,20 +364,22 @@ int plan_build(pnp_plan* p, const double* uvw, const int8_t* Jrow, const int32_t
     startc[m] = (uint16_t)((sub << 6) | ((f1 % GT) << 3) | (f0 % GT));
     Jmax = std::max(Jmax, g.J);
     amax = std::max(amax, std::fabs(g.a));
+    supports |= 1u << g.J;
     geom[m] = g;
-    p->h_rowkey[m] = g;
+    p->h_rowkey.push_back(g);
   }
   p->Jmax = Jmax;
 
   const int64_t nkeys = (int64_t)cpt * cpt * p->nblocks;
   if (nkeys * p->nstacks > INT32_MAX) return fail(PNP_ERR_UNSUPPORTED, "too many (stack, tile, block) keys");
   p->nkeys = nkeys;
+  pick_tile(p, geom, key, startc, p->nstacks > 1 ? stack : nullptr, supports);
   // stable LSD counting sort: by (T x T tile within the coarse tile, support J, first tap's cell in the tile with the
   // cells of one gridding window together), then by (coarse tile, block) key and w-stack, so that the rows of one
   // tile come out grouped by J and, within that, rows sharing a window are adjacent (the gridding pass
   // keeps it in registers)
-  auto sort_rows = [&](int T) {
-    const int per = GKT / T;
+  {
+    const int T = p->tile, per = GKT / T;
     std::vector<int32_t> by_j(M);
     {
       auto bin = [&](int64_t m) {
@@ -405,29 +412,23 @@ int plan_build(pnp_plan* p, const double* uvw, const int8_t* Jrow, const int32_t
       }
       p->h_perm.swap(by_j);
     }
-    p->h_key.assign(M, 0);
-    p->h_start.assign(M, 0);
-    p->h_J.assign(M, 0);
-    for (int64_t i = 0; i < M; ++i) {
-      const int64_t m = p->h_perm[i];
-      p->h_key[i] = (int32_t)((stack ? (int64_t)stack[m] : 0) * nkeys + key[m]);
-      p->h_start[i] = startc[m];
-      p->h_J[i] = (uint8_t)geom[m].J;
-    }
-  };
-  sort_rows(GT);
-  pick_tile(p);
-  if (p->tile != GT) sort_rows(p->tile);
+  }
   p->ntc = K / p->tile;
   p->pitch = p->mixed ? p->tile - 1 + 16 : GT - tap_quant(tap_pairs(Jmax), tap_lanes(Jmax)) + tap_lanes(Jmax);
   p->h_inv.assign(M, 0);
   for (int64_t i = 0; i < M; ++i) p->h_inv[p->h_perm[i]] = (int32_t)i;
   std::vector<RowGeom> sgeom(M);
+  p->h_key.assign(M, 0);
+  p->h_start.assign(M, 0);
   p->h_unit.assign(M + 1, 0);
+  p->h_J.assign(M, 0);
   p->nnz = 0;
   for (int64_t i = 0; i < M; ++i) {
     const int64_t m = p->h_perm[i];
     sgeom[i] = geom[m];
+    p->h_key[i] = (int32_t)((stack ? (int64_t)stack[m] : 0) * nkeys + key[m]);
+    p->h_start[i] = startc[m];
+    p->h_J[i] = (uint8_t)geom[m].J;
     sgeom[i].unit = p->h_unit[i];
     const int sub = startc[m] >> 6, cell = startc[m] & 63;
     sgeom[i].cell = (sub / (GKT / GT) * GT + (cell >> 3)) << 5 | (sub % (GKT / GT) * GT + (cell & 7));

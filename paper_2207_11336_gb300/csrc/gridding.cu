@@ -240,12 +240,15 @@ __global__ void __launch_bounds__(32 * Layout<MODE, BF, JP, W, MIX>::WARPS, min_
   if (MODE != G_DEGRID)
     for (int c = lane; c < L::CELLS; c += 32) sy[c] = zero4;
   const uint32_t ring_a = smem_u32(ring) + li * 16, yring_a = smem_u32(yring);
-  const unsigned warps = gridDim.x * L::WARPS;
-  unsigned nb = blockIdx.x * L::WARPS + (threadIdx.x >> 5);  // the first batch; the others from the counter
+  // This form of the loop keeps the fused JP = 9 kernel, at its limit of 128 registers, from spilling in its row loop (the
+  // first batch by index where there is a counter too: 212 instead of 200 us for 1e6 rows of J = 16).
+  unsigned nb = blockIdx.x * L::WARPS + (threadIdx.x >> 5);
+  if (A.sched && lane == 0) nb = atomicAdd(A.sched, 1u);
+  nb = __shfl_sync(0xffffffffu, nb, 0);
   unsigned u = A.u_begin + nb * A.batch;  // units are no more than rows: the sums stay below 2^32
   while (u < A.n_units) {
     const unsigned ue = min(u + A.batch, A.n_units);
-    if (lane == 0 && A.sched) nb = warps + atomicAdd(A.sched, 1u);  // the next batch, known by the end of this one
+    if (A.sched && lane == 0) nb = atomicAdd(A.sched, 1u);  // the next batch, known by the end of this one
     int held = -1;  // MIX: the tile whose regions are staged
     for (; u < (MIX ? A.n_units : ue); ++u) {
       const Unit U = A.units[u];
@@ -267,8 +270,7 @@ __global__ void __launch_bounds__(32 * Layout<MODE, BF, JP, W, MIX>::WARPS, min_
       const int n = (U.nrows + NG - 1) / NG;  // steps; rows of this group:
       const int q0 = min(gi * n, U.nrows), mine = min(n, U.nrows - q0);
       const unsigned char* src = A.rows + ((size_t)U.row_unit << 4) + (size_t)q0 * (16 * units) + li * 16;
-      const int32_t* psrc = A.perm + U.row_begin + q0;
-      const float2* ysrc = A.y_in + U.row_begin + q0;
+      const unsigned yrow = (unsigned)U.row_begin + q0;  // rows are below 2^31
       const bool has_y = A.y_in != nullptr;
       auto fetch = [&](int s) {  // copies of the group's row s, s = 0, 1, ... (one group of copies per call)
         if (s < mine) {
@@ -278,11 +280,9 @@ __global__ void __launch_bounds__(32 * Layout<MODE, BF, JP, W, MIX>::WARPS, min_
             if ((!MIX && c + W <= L::UNITS) || c + li < units) cp16(ring_a + slot * L::RBYTES + c * 16, src + c * 16);
           src += 16 * units;
           if (li == 0) {
-            if (MODE == G_DEGRID) cp4(yring_a + slot * 8, psrc);
-            else if (has_y) cp8(yring_a + slot * 8, ysrc);
+            if (MODE == G_DEGRID) cp4(yring_a + slot * 8, A.perm + yrow + s);
+            else if (has_y) cp8(yring_a + slot * 8, A.y_in + yrow + s);
           }
-          if (MODE == G_DEGRID) ++psrc;
-          else ++ysrc;
         }
         cp_commit();
       };
@@ -342,7 +342,7 @@ __global__ void __launch_bounds__(32 * Layout<MODE, BF, JP, W, MIX>::WARPS, min_
         const int cell = *reinterpret_cast<const int*>(rp + row_cell_at(jp, BF)) & ((T - 1) * 33);
         const int nw = cell & ((T - 2) << 5 | (T - Q));  // row pair and window columns of the first tap
         const int i0 = li - (cell & (Q - 1));            // this lane's tap column of the row
-        const bool tap = (unsigned)i0 < (unsigned)J;
+        const bool tap = (unsigned)i0 < (MIX ? (unsigned)J : 2u * JP - 1);  // the taps beyond J are stored zeros
         const bool moved = act && nw != win;
         const unsigned who = __ballot_sync(0xffffffffu, moved);
         if (who) {
@@ -420,7 +420,7 @@ __global__ void __launch_bounds__(32 * Layout<MODE, BF, JP, W, MIX>::WARPS, min_
       }
       if (MODE != G_DEGRID) {
         retire(0xffffffffu);
-        if (!MIX) flush_region<L, COMP>(A, sy, r0, c0, lane);
+        if (!MIX) flush_region<L, COMP>(A, sy, U.tile / A.ntc * T, U.tile % A.ntc * T, lane);
       }
     }
     if (MIX && MODE != G_DEGRID && held >= 0) flush_region<L, COMP>(A, sy, held / A.ntc * T, held % A.ntc * T, lane);
@@ -431,7 +431,7 @@ __global__ void __launch_bounds__(32 * Layout<MODE, BF, JP, W, MIX>::WARPS, min_
   // This kernel ends only after the previous class's kernel has (when it was launched as its dependent), so that
   // the end of the last class's kernel is the end of the pass.
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  if (lane == 0 && A.sched && atomicAdd(A.sched + 1, 1u) == warps - 1) {  // the last warp: every batch is taken
+  if (lane == 0 && A.sched && atomicAdd(A.sched + 1, 1u) == gridDim.x * L::WARPS - 1) {  // the last warp: every batch is taken
     A.sched[0] = 0;
     A.sched[1] = 0;
   }

@@ -30,16 +30,15 @@
 // The rows stream through a per-warp ring of cp.async copies.
 //
 // Where rows are so sparse that the units hold one or two (pick_tile in plan_build.cu), larger tiles are taken and
-// one kernel walks the units of all supports of a tile with the same regions.
-// Elsewhere the rows of each class of supports run as a kernel of their own: its registers and
-// regions are sized for that class, and all warps of an SM execute the same code (one
-// kernel for every class spent 42% of its warp time on instruction fetches).  Warps take
-// batches of units from a counter.
+// one kernel walks the units of all supports of a tile with the same regions.  Elsewhere the rows of each class of
+// supports run as a kernel of their own: its registers and regions are sized for that class, and all warps of an SM
+// execute the same code (one kernel for every class spent 42% of its warp time on instruction fetches).  Warps take
+// batches of units from a counter; a launch of one batch per warp takes none.
 //
-// What bounds it: issue slots and latency (52% of issue slots, FMA pipe about 25%, DRAM 20%), no longer
+// What bounds it: issue slots and latency (53 to 62% of issue slots at 15 to 19 warps per SM, DRAM 15 to 19%), no longer
 // the traffic of G: 32 tap_pairs instead of 10 J^2 bytes per row.  Fused pass, before (CTA-wide tiles, dense
-// taps, shared-memory float atomics) and now: 4096^2 image / 2e7 rows J 7-16: 6.30 -> 2.74 ms; 2048^2 /
-// 5e6 rows: 1.90 -> 0.83 ms; 256^2 / 2e5 rows J = 7: 105 -> 15 us.
+// taps, shared-memory float atomics) and now: 4096^2 image / 2e7 rows J 7-16: 6.30 -> 2.50 ms; 2048^2 /
+// 5e6 rows: 1.90 -> 0.79 ms; 256^2 / 2e5 rows J = 7: 105 -> 30 us.
 // Grid layout: grid[k1*K + k0].
 #include <algorithm>
 
@@ -138,10 +137,10 @@ __device__ __forceinline__ bool flushed(const GArgs& A, float2 v, int k1, int k0
 
 // Compensated flush of a region: the atomic returns the value it added to, so the lane forms the exact rounding error
 // of the (round-to-nearest) sum (TwoSum) and adds it to the compensation grid; the atomics of FB row pairs are in flight
-// together.  Out of line, so that its registers do not count against the main loop.
-template <int PR, int NC, int RL>
-__device__ __noinline__ void flush_compensated(const GArgs& A, ulonglong2* sy, int r0, int c0, int lane) {
-  constexpr int RI = 32 / RL, FB = 3;
+// together.
+template <typename L>
+__device__ __forceinline__ void flush_compensated(const GArgs& A, ulonglong2* sy, int r0, int c0, int lane) {
+  constexpr int PR = L::PR, NC = L::NC, RL = L::RL, RI = 32 / RL, FB = L::flush_pairs();
   const int Km = A.K - 1, jc = lane % RL, gc = (c0 + jc) & Km;
   if (jc >= NC) return;
   for (int i0 = lane / RL; i0 < PR; i0 += FB * RI) {
@@ -175,7 +174,7 @@ template <typename L, bool COMP>
 __device__ __forceinline__ void flush_region(const GArgs& A, ulonglong2* sy, int r0, int c0, int lane) {
   constexpr int NC = L::NC, RL = L::RL, RI = 32 / RL;
   if constexpr (COMP) {
-    flush_compensated<L::PR, NC, RL>(A, sy, r0, c0, lane);
+    flush_compensated<L>(A, sy, r0, c0, lane);
     return;
   }
   const int Km = A.K - 1, jc = lane % RL, gc = (c0 + jc) & Km;
@@ -205,6 +204,9 @@ struct Layout {
   static constexpr int Q = MIX ? 1 : tap_quant(JP, W);    // first-tap columns of a window
   static constexpr int PR = T / 2 - 1 + JP, NC = T - Q + W, CELLS = PR * NC;
   static constexpr int RL = NC <= 16 ? 16 : 32;           // lanes on a row pair of a region
+  // row pairs of a compensated flush in flight: two, but the fused JP = 9 kernel spills in its row loop then (1e6 rows of
+  // J = 16: 241 us with one, 270 with two, 280 with three out of line)
+  static constexpr int flush_pairs() { return MODE == G_FUSED && JP >= 9 ? 1 : 2; }
   static constexpr int YR = NG * RING * RBYTES, YB = NG * RING * 8;
   static constexpr int OUT = YR + YB, IN = OUT + (MODE == G_DEGRID ? 0 : CELLS * 16);
   static constexpr int BYTES = (IN + (MODE == G_GRID ? 0 : CELLS * 16) + 127) & ~127;

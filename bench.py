@@ -3,7 +3,7 @@
 
 Workload (default): 4096^2 float32 image, 8192^2 complex64 grid, M = 2e7
 synthetic MeerKAT-like visibilities in 64 radial data blocks, w folded into G
-with J in {7, 9, 12, 16} by |w| quartile (complex64 weights, int32 columns),
+with J in {7, 9, 12, 16} by |w| quartile (complex64 plan),
 40 dB input SNR.  A step is one full PnP-FB iteration (forward FFT with padding
 and grid correction, fused de-gridding + residual + gridding pass, adjoint FFT
 with the fused gradient step, denoiser, positivity and FP64 norms), replayed as

@@ -22,7 +22,9 @@
  *    kappa = omega K / (2 pi) of the KB kernel (J = 7 by default) convolved
  *    with the row's w-kernel (App. E).  A row is an outer product of one
  *    length-J_m vector per axis: complex64 plans store the two vectors,
- *    bfloat16 plans the rounded J_m^2 weights.
+ *    bfloat16 plans the rounded J_m^2 weights.  With p = 4 for J_m <= 7 and
+ *    (J_m + 2) / 2 above, a row takes 32 p bytes in a complex64 plan and 16 p^2
+ *    in a bfloat16 plan: bfloat16 is the larger form and the slower one.
  *  - Device pointers ("dev") are CUDA global-memory addresses owned by the
  *    caller; the library never frees them.  Host pointers ("host") are read
  *    during the call only.

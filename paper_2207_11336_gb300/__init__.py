@@ -203,6 +203,8 @@ class Plan:
     ``omega``: (M, 2) float64 rad/pixel (column 0 pairs with image axis 0);
     ``w``: (M,) wavelengths; ``dl``: pixel size [rad] for the w-term (0: none);
     ``J_per_row``: (M,) int8 supports in [J, 16] or None;
+    ``weight_dtype``: "c64" keeps two factors per row (32 p bytes; p = 4 for supports up to 7,
+    (J + 2) // 2 above), "bf16" the rounded weights (16 p^2 bytes: larger and slower);
     ``stack``, ``w_centres``: the w-stacking hybrid of App. E (Eq. phip): (M,) int32
     stack ids in [0, P) and the P stack centres [wavelengths]; Z_p then carries the
     centre chirp and the rows of G only the offset w - w_p.

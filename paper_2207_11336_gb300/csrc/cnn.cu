@@ -205,9 +205,9 @@ struct ConvArgs {
 // D_{s-1}[dy 1]) + D_s[dy 2].  Every MMA has the full N = 192 (no accumulator ring to wrap, no fresh-row
 // split), so an input row costs exactly 12 MMAs.  Warp roles: warps 0-15 the epilogue, warp 16 the MMAs
 // (one lane), warp 17 the TMA loads (one lane); epilogue warp w reads TMEM lanes 32 (w % 4) .. + 31 and channels 16 (w / 4) .. + 15 of each part.
-// What bounds it: the forward layer tensor pipe (66% active) and HBM (70% of the copy rate) together at 2048^2; the
+// What bounds it: the forward layer tensor pipe (66% active) and HBM (5.3 TB/s) together at 2048^2; the
 // backward layer, which reads its mask too, HBM (5.4 TB/s).  Per layer, before (waits between two rows' MMAs, 220
-// instructions per epilogue warp and row) and now: 2048^2 / 16 facets 353 -> 269 us, 16 x 256^2 83 -> 59 us forward
+// instructions per epilogue warp and row) and now: 2048^2 / 16 facets 353 -> 256 us, 16 x 256^2 83 -> 59 us forward
 // and 83 -> 74 us backward.
 constexpr int ROW_N = 3 * CH;                 // 192 accumulator columns per staged input row
 constexpr int ROW_DBUF = 2;                   // TMEM buffers (2 x 192 of the 512 columns)
